@@ -160,8 +160,8 @@ cudaError_t launch_ctx_step_fp64(pond_ctx* ctx, const StateBuf<double>& in,
     if (ctx_staged(ctx))
         return launch_step_staged_fp64(in, out, iters, stats, ctx->grids_dev, ctx->tile_prefix_dev,
                                        ctx->n_grids, ctx->n_tiles, ctx->N,
-                                       ctx->n_grids > 1 ? ctx->work_counter : nullptr, ctx->win,
-                                       ctx->persistent_ctas, ctx->L, ctx->P, ctx->stream);
+                                       ctx->n_grids > 1 ? ctx->work_counter : nullptr, ctx->redo,
+                                       ctx->win, ctx->persistent_ctas, ctx->L, ctx->P, ctx->stream);
     const GridDesc& G = ctx->grids_host[0];
     return launch_step_fp64(in, out, iters, stats, G.nx, G.ny, ctx->L, ctx->P, fp64_npw(ctx),
                             ctx->stream);
@@ -414,6 +414,15 @@ pond_status pond_create(const pond_config* cfg, int32_t n_grids, const int32_t* 
     ok = ok && alloc((void**)&ctx->tile_prefix_dev, sizeof(int64_t) * (n_grids + 1), "alloc prefix");
     ok = ok && alloc((void**)&ctx->work_counter, sizeof(unsigned int), "alloc counter");
     ok = ok && alloc((void**)&ctx->bounds_dev, 8 * sizeof(float), "alloc bounds");
+    size_t redo_words = 0;
+    if (!mixed(ctx) && ctx_staged(ctx)) {
+        // two counters and the tiles of the finest FP64 shape
+        redo_words = 2;
+        for (int g = 0; g < n_grids; ++g)
+            redo_words += ((size_t)(nx[g] + MIXED_TX - 1) / MIXED_TX) *
+                          (((size_t)ny[g] + STAGED_TY_FP64[0] - 1) / STAGED_TY_FP64[0]);
+        ok = ok && alloc((void**)&ctx->redo, sizeof(unsigned int) * redo_words, "alloc redo list");
+    }
     if (ok) {
         cudaError_t e = cudaMallocHost((void**)&ctx->stats_host, sizeof(DevStats));
         if (e != cudaSuccess) {
@@ -426,6 +435,7 @@ pond_status pond_create(const pond_config* cfg, int32_t n_grids, const int32_t* 
                                    sizeof(GridDesc) * n_grids, cudaMemcpyHostToDevice);
 
         if (e == cudaSuccess) e = cudaMemset(ctx->iters, 0, sizeof(int32_t) * ctx->N);
+        if (e == cudaSuccess && ctx->redo) e = cudaMemset(ctx->redo, 0, 2 * sizeof(unsigned int));
         if (e == cudaSuccess) e = upload_lattice_fp64();
         if (e == cudaSuccess) e = upload_lattice_mixed();
         if (e == cudaSuccess) e = upload_lattice_adjoint();
@@ -865,6 +875,7 @@ void pond_destroy(pond_ctx* ctx) {
     cudaFree(ctx->grids_dev);
     cudaFree(ctx->tile_prefix_dev);
     cudaFree(ctx->work_counter);
+    cudaFree(ctx->redo);
     cudaFree(ctx->bounds_dev);
     cudaFree(ctx->staging);
     if (ctx->stats_host) cudaFreeHost(ctx->stats_host);

@@ -197,10 +197,12 @@ cudaError_t launch_step_mixed(const StateBuf<float>& in, const StateBuf<float>& 
 // forms, over one or many grids (tiles 32 x ty; ty 4 or 8 in FP64, 4, 8 or
 // 16 in the mixed form), its per-device set-up (returns resident CTAs per SM
 // for a dynamic shared-memory size) and that size for a window.
+// redo: the FP64 form's {count, exit count, tile list} of n_tiles + 2 words,
+// the first two zero before the first launch (each launch leaves them zero).
 cudaError_t launch_step_staged_fp64(const StateBuf<double>& in, const StateBuf<double>& out,
                                     int32_t* iters, DevStats* stats, const GridDesc* grids_dev,
                                     const int64_t* tile_prefix_dev, int n_grids, int64_t n_tiles,
-                                    int64_t plane, unsigned int* work_counter,
+                                    int64_t plane, unsigned int* work_counter, unsigned int* redo,
                                     const TileWindow& win, int persistent_ctas, const Lattice& L,
                                     const StepParams& P, cudaStream_t s);
 cudaError_t launch_step_staged_mixed(const StateBuf<float>& in, const StateBuf<float>& out,
@@ -304,6 +306,7 @@ struct pond_ctx {
     pond::GridDesc* grids_dev = nullptr;
     int64_t* tile_prefix_dev = nullptr;
     unsigned int* work_counter = nullptr;
+    unsigned int* redo = nullptr;  // staged FP64 step: tiles left to the FP64 kernel
     float* bounds_dev = nullptr;
     int64_t n_tiles = 0;
     int tile_ty = pond::MIXED_TY;  // rows of the mixed kernel's tile

@@ -47,9 +47,9 @@
 //
 // Tr (the including translation unit's traits) provides:
 //   Real, Real4 (16 or 32 bytes), kUnrollK, kPacked (the packed FP32 sweep),
-//   kEyTable (the Ey table in shared memory), min_blocks<threads>(),
-//   lat<N1>() (lattice constants of that unit's constant bank), departure
-//   (the floor of a displacement and the cubic weights at its fraction),
+//   kRedo (the kernel runs k_step_fixed's left-over tiles), kEyTable (the Ey
+//   table in shared memory), min_blocks<threads>(), lat<N1>() (lattice constants of that unit's
+//   constant bank), departure (the floor of a displacement and the cubic weights at its fraction),
 //   load4 / store4, update(...) (the moments -> gauge update and the App. E
 //   test of that form) and finish<N1>(...) (re-gauge into the co-moving
 //   frame, BGK, store).
@@ -75,6 +75,10 @@ struct StagedArgs {
     long long n_tiles;
     long long plane;  // plane stride of the packed state
     unsigned int* work_counter;
+    // tiles k_step_fixed left to k_step_staged<StagedFP64>: {count, CTAs of the
+    // redo launch that have exited}, and the tiles (FP64 form only)
+    unsigned int* redo_count;
+    unsigned int* redo_list;
     int ww, wh;       // allocated window
     double c_max;
     float margin;
@@ -276,8 +280,16 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
     const unsigned long long t_begin = (A.work_counter && tid == 0) ? pond_globaltimer() : 0ull;
 
     long long item = blockIdx.x;
+    // the redo launch takes its tiles from the list k_step_fixed left
+    const bool redo = Tr::kRedo && A.redo_count != nullptr;
+    unsigned int redo_i = blockIdx.x;
+    const unsigned int redo_n = redo ? *A.redo_count : 0u;
     for (;;) {
-        if (A.work_counter) {
+        if (redo) {
+            if (redo_i >= redo_n) break;
+            item = A.redo_list[redo_i];
+            redo_i += gridDim.x;
+        } else if (A.work_counter) {
             __syncthreads();
             if (tid == 0) s_item = (long long)atomicAdd(A.work_counter, 1u);
             __syncthreads();
@@ -638,17 +650,26 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
             if (pg.flag & 2u) atomicAdd(&s_np, 1ull);
             if (fallbacks) atomicAdd(&s_fb, (unsigned long long)fallbacks);
         }
-        if (!A.work_counter) break;
+        if (!A.work_counter && !redo) break;
         __syncthreads();  // the next item restages the window
     }
     __syncthreads();
-    if (tid == 0 && A.stats) {
+    if (tid == 0 && A.stats && !(redo && redo_n == 0u)) {
         atomicAdd(&A.stats->passes, s_passes);
         atomicMax(&A.stats->max_passes, s_max);
         if (s_nc) atomicAdd(&A.stats->nonconverged, s_nc);
         if (s_np) atomicAdd(&A.stats->nonphysical, s_np);
         if (s_fb) atomicAdd(&A.stats->halo_fallback, s_fb);
-        if (A.work_counter) persistent_exit(A.stats, t_begin);
+        if (A.work_counter && !redo) persistent_exit(A.stats, t_begin);
+    }
+    // the redo launch's last CTA clears the list for the next step (every
+    // CTA has read the count by then)
+    if (redo && tid == 0) {
+        __threadfence();
+        if (atomicAdd(A.redo_count + 1, 1u) == gridDim.x - 1) {
+            A.redo_count[0] = 0u;
+            A.redo_count[1] = 0u;
+        }
     }
 }
 

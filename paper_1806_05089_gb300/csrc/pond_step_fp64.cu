@@ -41,7 +41,7 @@
 #include <mutex>
 
 #include "pond_device.cuh"
-#include "pond_staged.cuh"
+#include "pond_fixed.cuh"
 
 namespace pond {
 
@@ -570,6 +570,7 @@ struct StagedFP64 {
     using Real4 = Double4;
     static constexpr bool kUnrollK = true;
     static constexpr bool kPacked = false;  // the sweep on packed FP32 pairs
+    static constexpr bool kRedo = true;
     // the y-map entries Ey[l][b] of a pass in a shared-memory table (they do
     // not depend on the x-speed; computing them once per pass instead of once
     // per (k, l) saves ~190 FP64 operations per node-pass)
@@ -709,11 +710,16 @@ struct StagedFP64 {
     }
 };
 
+// The fixed-point kernel and the FP64 kernel of its left-over tiles share
+// one shared-memory layout size; the resident CTAs are the fixed-point one's.
 template <int TY, int N1>
 static cudaError_t staged64_shape(size_t smem, int* per_sm, int* s_set) {
-    void (*kern)(StagedArgs<double>) = k_step_staged<StagedFP64, 32, TY, N1>;
+    void (*kern)(StagedArgs<double>) = k_step_fixed<StagedFP64, TY, N1>;
+    void (*left)(StagedArgs<double>) = k_step_staged<StagedFP64, 32, TY, N1>;
     if ((int)smem > *s_set) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(left, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         *s_set = (int)smem;
     }
@@ -738,11 +744,11 @@ cudaError_t staged_prepare_fp64(int ty, int n1, size_t smem, int* ctas_per_sm) {
 cudaError_t launch_step_staged_fp64(const StateBuf<double>& in, const StateBuf<double>& out,
                                     int32_t* iters, DevStats* stats, const GridDesc* grids_dev,
                                     const int64_t* tile_prefix_dev, int n_grids, int64_t n_tiles,
-                                    int64_t plane, unsigned int* work_counter,
+                                    int64_t plane, unsigned int* work_counter, unsigned int* redo,
                                     const TileWindow& win, int persistent_ctas, const Lattice& L,
                                     const StepParams& P, cudaStream_t s) {
     if (n_tiles == 0) return cudaSuccess;
-    if (win.n1 != L.n1 || (win.ty != 4 && win.ty != 8) || win.tx != 32) return cudaErrorInvalidValue;
+    if (!redo || win.n1 != L.n1 || (win.ty != 4 && win.ty != 8) || win.tx != 32) return cudaErrorInvalidValue;
     StagedArgs<double> A{};
     A.in = in;
     A.out = out;
@@ -754,6 +760,8 @@ cudaError_t launch_step_staged_fp64(const StateBuf<double>& in, const StateBuf<d
     A.n_tiles = n_tiles;
     A.plane = plane;
     A.work_counter = work_counter;
+    A.redo_count = redo;
+    A.redo_list = redo + 2;
     A.ww = win.ww;
     A.wh = win.wh;
     A.c_max = L.c_max;
@@ -768,6 +776,15 @@ cudaError_t launch_step_staged_fp64(const StateBuf<double>& in, const StateBuf<d
     } else {
         nb = (unsigned int)n_tiles;
     }
+    if (L.n1 == 3) {
+        if (win.ty == 4) k_step_fixed<StagedFP64, 4, 3><<<nb, 128, smem, s>>>(A);
+        else k_step_fixed<StagedFP64, 8, 3><<<nb, 256, smem, s>>>(A);
+    } else {
+        if (win.ty == 4) k_step_fixed<StagedFP64, 4, 4><<<nb, 128, smem, s>>>(A);
+        else k_step_fixed<StagedFP64, 8, 4><<<nb, 256, smem, s>>>(A);
+    }
+    // the tiles out of the fixed-point form's range (usually none)
+    nb = (unsigned int)(persistent_ctas < n_tiles ? persistent_ctas : n_tiles);
     if (L.n1 == 3) {
         if (win.ty == 4) k_step_staged<StagedFP64, 32, 4, 3><<<nb, 128, smem, s>>>(A);
         else k_step_staged<StagedFP64, 32, 8, 3><<<nb, 256, smem, s>>>(A);
