@@ -48,11 +48,11 @@
 // Tr (the including translation unit's traits) provides:
 //   Real, Real4 (16 or 32 bytes), kUnrollK, kPacked (the packed FP32 sweep),
 //   kRedo (the kernel runs k_step_fixed's left-over tiles), kEyTable (the Ey
-//   table in shared memory), min_blocks<threads>(), lat<N1>() (lattice constants of that unit's
-//   constant bank), departure (the floor of a displacement and the cubic weights at its fraction),
-//   load4 / store4, update(...) (the moments -> gauge update and the App. E
-//   test of that form) and finish<N1>(...) (re-gauge into the co-moving
-//   frame, BGK, store).
+//   table in shared memory), min_blocks<threads>(), lat<N1>() (lattice
+//   constants of that unit's constant bank), departure (the floor of a
+//   displacement and the cubic weights at its fraction), load4 / store4,
+//   update(...) (the moments -> gauge update and the App. E test of that form)
+//   and finish<N1>(...) (re-gauge into the co-moving frame, BGK, store).
 #pragma once
 
 #include "pond_device.cuh"

@@ -50,10 +50,14 @@ constexpr int K1_WARPS = 4;
 // Lattice constants of this translation unit (uploaded once per device),
 // slot lattice_slot(N1).
 __constant__ Lattice c_L[2];
+__constant__ LatticeFix c_Lfix[2];
 
 cudaError_t upload_lattice_fp64() {
     const Lattice L[2] = {make_lattice(POND_D2Q16), make_lattice(POND_D2Q9)};
-    return cudaMemcpyToSymbol(c_L, L, sizeof(L));
+    const LatticeFix F[2] = {make_lattice_fix(L[0]), make_lattice_fix(L[1])};
+    cudaError_t e = cudaMemcpyToSymbol(c_L, L, sizeof(L));
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_Lfix, F, sizeof(F));
+    return e;
 }
 
 // NPW nodes per warp.  NPW = 1: lane = (q, half of the stencil rows), the
@@ -582,6 +586,10 @@ struct StagedFP64 {
     template <int N1>
     static __device__ __forceinline__ const Lattice& lat() {
         return c_L[lattice_slot(N1)];
+    }
+    template <int N1>
+    static __device__ __forceinline__ const LatticeFix& lat_fix() {
+        return c_Lfix[lattice_slot(N1)];
     }
     static __device__ __forceinline__ void lagrange(double t, double (&l)[4]) { lagrange4(t, l); }
     // floor of the displacement d and the cubic weights at t = d - floor + 1
