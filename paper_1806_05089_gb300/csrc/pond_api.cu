@@ -120,8 +120,10 @@ pond_status update_window(pond_ctx* ctx) {
     w.n1 = ctx->L.n1;
     w.staged = ctx_staged(ctx) ? 1 : 0;
     w.real_bytes = mixed(ctx) ? 4 : 8;
-    w.ww = w.tx + window_extent(sx, dt, 2 * margin) + 5;
-    w.wh = w.ty + window_extent(sy, dt, 2 * margin) + 5;
+    const int ex = window_extent(sx, dt, 2 * margin) + 5, ey = window_extent(sy, dt, 2 * margin) + 5;
+    w.ww = w.tx + ex;
+    w.wh = w.ty + ey;
+    w.fx = w.fy = w.fks = w.fww = w.fwh = 0;
     // cap the staged window at the shared memory a CTA can have; stencils
     // beyond it take the global-memory path
     auto bytes = [](const TileWindow& v) {
@@ -132,16 +134,15 @@ pond_status update_window(pond_ctx* ctx) {
         if (w.ww - w.tx >= w.wh - w.ty) --w.ww; else --w.wh;
     }
     const size_t smem = bytes(w);
-    int per_sm = 0;
+    int per_sm = 0, sms = 0;
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device), "SM count");
     if (!w.staged)
         CK(mixed_prepare(w.ty, w.pair != 0, w.n1, smem, &per_sm), "mixed kernel set-up");
     else if (mixed(ctx))
         CK(staged_prepare_mixed(w.ty, w.n1, smem, &per_sm), "staged kernel set-up");
     else
-        CK(staged_prepare_fp64(w.ty, w.n1, smem, &per_sm), "staged kernel set-up");
+        CK(staged_prepare_fp64(&w, ex, ey, ctx->n_tiles, sms, &per_sm), "staged kernel set-up");
     if (per_sm < 1) return fail(ctx, POND_ERR_CUDA, "tile kernel does not fit on an SM");
-    int sms = 0;
-    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device), "SM count");
     ctx->win = w;
     ctx->persistent_ctas = per_sm * sms;
     return POND_OK;
@@ -416,10 +417,10 @@ pond_status pond_create(const pond_config* cfg, int32_t n_grids, const int32_t* 
     ok = ok && alloc((void**)&ctx->bounds_dev, 8 * sizeof(float), "alloc bounds");
     size_t redo_words = 0;
     if (!mixed(ctx) && ctx_staged(ctx)) {
-        // two counters and the tiles of the finest FP64 shape
+        // two counters and the 8-node-wide parts of the finest FP64 tiles
         redo_words = 2;
         for (int g = 0; g < n_grids; ++g)
-            redo_words += ((size_t)(nx[g] + MIXED_TX - 1) / MIXED_TX) *
+            redo_words += 4 * (((size_t)nx[g] + MIXED_TX - 1) / MIXED_TX) *
                           (((size_t)ny[g] + STAGED_TY_FP64[0] - 1) / STAGED_TY_FP64[0]);
         ok = ok && alloc((void**)&ctx->redo, sizeof(unsigned int) * redo_words, "alloc redo list");
     }
@@ -561,7 +562,9 @@ pond_status pond_set_state(pond_ctx* ctx, int32_t grid, const void* rho, const v
     ctx->grid_set[grid] = 1;
     const TileWindow before = ctx->win;
     s = update_window(ctx);
-    if (before.ww != ctx->win.ww || before.wh != ctx->win.wh) drop_graphs(ctx);
+    if (before.ww != ctx->win.ww || before.wh != ctx->win.wh || before.fww != ctx->win.fww ||
+        before.fwh != ctx->win.fwh || before.fx != ctx->win.fx)
+        drop_graphs(ctx);
     return s;
 }
 

@@ -182,6 +182,10 @@ struct TileWindow {
     int n1;           // speeds per dimension of the lattice (4 or 3)
     int staged;       // 1: the reference-gauge staged kernel
     int real_bytes;   // 8 (FP64 form) or 4 (mixed form)
+    // the FP64 form's fixed-point kernel: its CTA's part of the tile, threads
+    // per node and staged window
+    int fx, fy, fks;
+    int fww, fwh;
 };
 
 // Mixed-precision step over one or many grids (one CTA per tile; batched
@@ -211,7 +215,11 @@ cudaError_t launch_step_staged_mixed(const StateBuf<float>& in, const StateBuf<f
                                      int64_t plane, unsigned int* work_counter,
                                      const TileWindow& win, int persistent_ctas, const Lattice& L,
                                      const StepParams& P, cudaStream_t s);
-cudaError_t staged_prepare_fp64(int ty, int n1, size_t smem, int* ctas_per_sm);
+// (FP64: completes the window with the fixed-point kernel's shape and staged
+// window, for velocity spreads that need ex x ey extra nodes, by the number of
+// 32 x ty tiles a step has)
+cudaError_t staged_prepare_fp64(TileWindow* win, int ex, int ey, int64_t n_tiles, int sms,
+                                int* ctas_per_sm);
 cudaError_t staged_prepare_mixed(int ty, int n1, size_t smem, int* ctas_per_sm);
 // Extra window extent, in nodes, that one step's departures need for a
 // particle-speed spread `span`: ceil(span * dt + pad), bounded by 65536 so

@@ -78,7 +78,8 @@ struct StagedArgs {
     // tiles k_step_fixed left to k_step_staged<StagedFP64>: {count, CTAs of the
     // redo launch that have exited}, and the tiles (FP64 form only)
     unsigned int* redo_count;
-    unsigned int* redo_list;
+    unsigned int* redo_list;  // entries tile * (sub_x * sub_y) + sub
+    int sub_x, sub_y;         // parts of a tile that k_step_fixed's CTAs take
     int ww, wh;       // allocated window
     double c_max;
     float margin;
@@ -283,12 +284,15 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
     // the redo launch takes its tiles from the list k_step_fixed left
     const bool redo = Tr::kRedo && A.redo_count != nullptr;
     unsigned int redo_i = blockIdx.x;
+    int redo_sub = 0;
     const unsigned int redo_n = redo ? *A.redo_count : 0u;
     for (;;) {
         if (redo) {
             if (redo_i >= redo_n) break;
             item = A.redo_list[redo_i];
             redo_i += gridDim.x;
+            redo_sub = (int)(item % (A.sub_x * A.sub_y));
+            item /= A.sub_x * A.sub_y;
         } else if (A.work_counter) {
             __syncthreads();
             if (tid == 0) s_item = (long long)atomicAdd(A.work_counter, 1u);
@@ -314,7 +318,10 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
         const int tx0 = G.ix0 + (int)(t % tiles_x) * TX;
         const int ty0 = G.iy0 + (int)(t / tiles_x) * TY;
         const int X = tx0 + lxi, Y = ty0 + lyi;
-        const bool valid = X < G.ix0 + G.iw && Y < G.iy0 + G.ih;
+        bool valid = X < G.ix0 + G.iw && Y < G.iy0 + G.ih;
+        if (redo)  // only the part of the tile that was left over
+            valid = valid && lxi / (TX / A.sub_x) == redo_sub % A.sub_x &&
+                    lyi / (TY / A.sub_y) == redo_sub / A.sub_x;
         const long long base = G.offset;
         const long long node = base + (long long)Y * G.nx + X;
 

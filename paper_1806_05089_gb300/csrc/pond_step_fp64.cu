@@ -718,35 +718,86 @@ struct StagedFP64 {
     }
 };
 
-// The fixed-point kernel and the FP64 kernel of its left-over tiles share
-// one shared-memory layout size; the resident CTAs are the fixed-point one's.
-template <int TY, int N1>
-static cudaError_t staged64_shape(size_t smem, int* per_sm, int* s_set) {
-    void (*kern)(StagedArgs<double>) = k_step_fixed<StagedFP64, TY, N1>;
-    void (*left)(StagedArgs<double>) = k_step_staged<StagedFP64, 32, TY, N1>;
-    if ((int)smem > *s_set) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(left, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        *s_set = (int)smem;
-    }
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, 32 * TY, smem);
+// Shapes of the fixed-point kernel: the part TXS x TYS of a 32 x TY tile that
+// a CTA takes, and the threads per node.
+struct FixedShape {
+    int n1, ty, fx, fy, ks;
+    void (*kern)(StagedArgs<double>);
+};
+template <int N1, int TY, int FX, int FY, int KS, int MINB>
+constexpr FixedShape fixed_shape() {
+    return {N1, TY, FX, FY, KS, k_step_fixed<StagedFP64, 32, TY, FX, FY, KS, N1, MINB>};
+}
+static const FixedShape kFixedShapes[] = {
+    fixed_shape<4, 8, 32, 8, 1, 1>(), fixed_shape<4, 8, 16, 8, 1, 2>(), fixed_shape<4, 8, 8, 8, 4, 1>(),
+    fixed_shape<4, 4, 32, 4, 1, 2>(), fixed_shape<4, 4, 8, 4, 4, 2>(),
+    fixed_shape<3, 8, 32, 8, 1, 1>(), fixed_shape<3, 8, 8, 8, 4, 1>(),
+    fixed_shape<3, 4, 32, 4, 1, 2>(), fixed_shape<3, 4, 8, 4, 4, 2>(),
+};
+constexpr int kFixedShapeCount = sizeof(kFixedShapes) / sizeof(kFixedShapes[0]);
+
+static void (*staged64_kernel(int ty, int n1))(StagedArgs<double>) {
+    if (n1 == 3) return ty == 4 ? k_step_staged<StagedFP64, 32, 4, 3> : k_step_staged<StagedFP64, 32, 8, 3>;
+    return ty == 4 ? k_step_staged<StagedFP64, 32, 4, 4> : k_step_staged<StagedFP64, 32, 8, 4>;
 }
 
-cudaError_t staged_prepare_fp64(int ty, int n1, size_t smem, int* ctas_per_sm) {
-    static int s_set[64][4] = {{0}};
+static size_t fixed_bytes(const TileWindow& w) {
+    return fixed_smem_bytes(w.n1, w.fww, w.fwh, w.fx * w.fy);
+}
+
+// The attribute is per function and device: only ever raised, so that every
+// live context's window stays launchable.
+static cudaError_t raise_smem(void (*kern)(StagedArgs<double>), size_t smem, int* set) {
+    if ((int)smem <= *set) return cudaSuccess;
+    const cudaError_t e =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) *set = (int)smem;
+    return e;
+}
+
+cudaError_t staged_prepare_fp64(TileWindow* win, int ex, int ey, int64_t n_tiles, int sms,
+                                int* ctas_per_sm) {
+    static int s_left[64][4] = {{0}}, s_fixed[64][kFixedShapeCount] = {{0}};
+    const int ty = win->ty, n1 = win->n1;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    const int slot = (n1 == 3 ? 2 : 0) + (ty == 8 ? 1 : 0);
     if (ty != 4 && ty != 8) return cudaErrorInvalidValue;
-    if (n1 == 3)
-        return ty == 4 ? staged64_shape<4, 3>(smem, ctas_per_sm, &s_set[dev][slot])
-                       : staged64_shape<8, 3>(smem, ctas_per_sm, &s_set[dev][slot]);
-    return ty == 4 ? staged64_shape<4, 4>(smem, ctas_per_sm, &s_set[dev][slot])
-                   : staged64_shape<8, 4>(smem, ctas_per_sm, &s_set[dev][slot]);
+    e = raise_smem(staged64_kernel(ty, n1), staged_window_bytes(*win),
+                   &s_left[dev][(n1 == 3 ? 2 : 0) + (ty == 8 ? 1 : 0)]);
+    if (e != cudaSuccess) return e;
+    // Narrower parts than the whole tile when the tiles do not fill the chip (8
+    // wide, four lanes per node; 64^2: 373 -> 131 us a step, 160^2 with 100
+    // tiles: 335 -> 321, with 144 tiles slower), or, on D2Q16, where one CTA of
+    // the tile fills an SM, when the last wave is at most half full (a half costs
+    // 0.53 of a tile, for its wider share of halo; 168 tiles: 555 -> 473 us)
+    const int64_t waves = (n_tiles + sms - 1) / sms, half_waves = (2 * n_tiles + sms - 1) / sms;
+    const bool halves = n1 == 4 && ty == 8 && 53 * half_waves < 100 * waves;
+    const int widest = 3 * n_tiles <= 2 * sms ? 8 : halves ? 16 : 32;
+    const size_t cap = 225 * 1024;
+    int pick = -1;
+    for (int i = 0; i < kFixedShapeCount; ++i) {
+        const FixedShape& f = kFixedShapes[i];
+        if (f.n1 != n1 || f.ty != ty) continue;
+        if (f.fx > widest) continue;
+        pick = i;
+        win->fx = f.fx;
+        win->fy = f.fy;
+        win->fks = f.ks;
+        win->fww = f.fx + ex;
+        win->fwh = f.fy + ey;
+        if (fixed_bytes(*win) <= cap) break;
+    }
+    if (pick < 0) return cudaErrorInvalidValue;
+    while (fixed_bytes(*win) > cap) {
+        if (win->fww - win->fx >= win->fwh - win->fy) --win->fww; else --win->fwh;
+    }
+    const FixedShape& f = kFixedShapes[pick];
+    e = raise_smem(f.kern, fixed_bytes(*win), &s_fixed[dev][pick]);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, f.kern, f.fx * f.fy * f.ks,
+                                                         fixed_bytes(*win));
 }
 
 cudaError_t launch_step_staged_fp64(const StateBuf<double>& in, const StateBuf<double>& out,
@@ -770,36 +821,32 @@ cudaError_t launch_step_staged_fp64(const StateBuf<double>& in, const StateBuf<d
     A.work_counter = work_counter;
     A.redo_count = redo;
     A.redo_list = redo + 2;
-    A.ww = win.ww;
-    A.wh = win.wh;
+    A.sub_x = win.tx / win.fx;
+    A.sub_y = win.ty / win.fy;
+    A.ww = win.fww;
+    A.wh = win.fwh;
     A.c_max = L.c_max;
     A.margin = 1.0f;
     A.P = P;
-    const size_t smem = staged_smem_bytes(L.n1, win.ww, win.wh, 32 * win.ty, sizeof(double));
-    unsigned int nb;
+    const FixedShape* f = nullptr;
+    for (const FixedShape& c : kFixedShapes)
+        if (c.n1 == L.n1 && c.ty == win.ty && c.fx == win.fx && c.fy == win.fy && c.ks == win.fks) f = &c;
+    if (!f) return cudaErrorInvalidValue;
+    const int64_t parts = n_tiles * A.sub_x * A.sub_y;
+    unsigned int nb = (unsigned int)parts;
     if (work_counter) {
         cudaError_t e = cudaMemsetAsync(work_counter, 0, sizeof(unsigned int), s);
         if (e != cudaSuccess) return e;
-        nb = (unsigned int)(persistent_ctas < n_tiles ? persistent_ctas : n_tiles);
-    } else {
-        nb = (unsigned int)n_tiles;
+        if (persistent_ctas < parts) nb = (unsigned int)persistent_ctas;
     }
-    if (L.n1 == 3) {
-        if (win.ty == 4) k_step_fixed<StagedFP64, 4, 3><<<nb, 128, smem, s>>>(A);
-        else k_step_fixed<StagedFP64, 8, 3><<<nb, 256, smem, s>>>(A);
-    } else {
-        if (win.ty == 4) k_step_fixed<StagedFP64, 4, 4><<<nb, 128, smem, s>>>(A);
-        else k_step_fixed<StagedFP64, 8, 4><<<nb, 256, smem, s>>>(A);
-    }
+    f->kern<<<nb, f->fx * f->fy * f->ks, fixed_bytes(win), s>>>(A);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     // the tiles out of the fixed-point form's range (usually none)
+    A.ww = win.ww;
+    A.wh = win.wh;
     nb = (unsigned int)(persistent_ctas < n_tiles ? persistent_ctas : n_tiles);
-    if (L.n1 == 3) {
-        if (win.ty == 4) k_step_staged<StagedFP64, 32, 4, 3><<<nb, 128, smem, s>>>(A);
-        else k_step_staged<StagedFP64, 32, 8, 3><<<nb, 256, smem, s>>>(A);
-    } else {
-        if (win.ty == 4) k_step_staged<StagedFP64, 32, 4, 4><<<nb, 128, smem, s>>>(A);
-        else k_step_staged<StagedFP64, 32, 8, 4><<<nb, 256, smem, s>>>(A);
-    }
+    staged64_kernel(win.ty, L.n1)<<<nb, 32 * win.ty, staged_window_bytes(win), s>>>(A);
     return cudaGetLastError();
 }
 

@@ -11,7 +11,7 @@ import numpy as np
 import pytest
 
 import oracle
-from paper_1806_05089_gb300 import pond, workloads
+from paper_1806_05089_gb300 import decomp, pond, workloads
 
 pytestmark = pytest.mark.gpu
 
@@ -71,3 +71,34 @@ def test_scaled_populations_scale_the_result_exactly(power):
     b, _ = run(fields, 2, f=np.ldexp(f, power))
     assert np.array_equal(np.ldexp(a.f, power), b.f)
     assert np.array_equal(a.ux, b.ux) and np.array_equal(a.T, b.T)
+
+
+@pytest.mark.parametrize("lattice,tile_rows,nx,ny,px,py", [
+    (pond.POND_D2Q16, 8, 512, 160, 2, 2),   # 320 whole tiles against 80 by parts of 8
+    (pond.POND_D2Q16, 8, 256, 176, 1, 2),   # 176 half tiles against 88 by parts
+    (pond.POND_D2Q16, 4, 256, 128, 2, 2),   # 256 against 64, four rows
+    (pond.POND_D2Q9, 8, 512, 160, 2, 2), (pond.POND_D2Q9, 4, 256, 128, 2, 2)])
+def test_parts_of_tiles_match_whole_tiles_bit_for_bit(lattice, tile_rows, nx, ny, px, py):
+    T_L = 1.0 / 3.0 if lattice == pond.POND_D2Q9 else 1.0
+    fields = field("plain", nx, ny, T_L)
+    cfg = dict(lattice=lattice, T_ref=T_L)
+    whole, _ = run(fields, 2, tile_rows=tile_rows, **cfg)
+    with decomp.DecomposedSim(nx, ny, px, py, 14, precision=pond.POND_FP64, tile_rows=tile_rows,
+                              **cfg) as d:
+        d.set_state(fields.rho, fields.ux, fields.uy, fields.T)
+        d.step(2)
+        f, g = d.gather_state()
+    assert np.array_equal(whole.f, f)
+    for a, b in zip((whole.ux, whole.uy, whole.T), g):
+        assert np.array_equal(a, b)
+
+
+def test_a_window_too_large_for_whole_tiles_runs_by_halves():
+    """T = 6: the staged window of a 32 x 8 tile exceeds the shared memory."""
+    fields = field("plain", 640, 200, 1.0)
+    fields.T = 6.0 * fields.T
+    a, _ = run(fields, 1, fixed_iter=4)
+    b, _ = run(fields, 1, fixed_iter=4, kernel=pond.POND_KERNEL_DIRECT)
+    assert np.abs(a.f - b.f).max() <= TOL64 * np.abs(b.f).max()
+    assert np.abs(a.ux - b.ux).max() <= TOL64 * np.sqrt(6.0)
+    assert np.max(np.abs(a.T - b.T) / b.T) <= TOL64
