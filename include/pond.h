@@ -347,8 +347,12 @@ pond_status pond_max_displacement(pond_ctx* ctx, int32_t grid, double* out);
  * so calls whose work can overlap on the GPU (different streams, or
  * different host threads) race and must be serialised by the caller.  Every
  * call looks up the array's device address (a lookup, not an allocation).
- * The first call in each CUDA context also uploads the lattice constants (a
- * synchronous copy), so make it before any stream capture; after a device
+ * The step is the staged kernel's, as pond_create's default (its windows are
+ * sized by the shared memory instead of the velocities); nodes_per_warp != 0
+ * or kernel = POND_KERNEL_DIRECT select the direct kernels, tile_rows is
+ * ignored.  The first call in each CUDA context also uploads the lattice
+ * constants (a synchronous copy) and launches each of the step's kernels over
+ * no tiles, so make it before any stream capture; after a device
  * reset the next call sees the new context and uploads them again.  With
  * lazy module loading (the CUDA default) the driver loads this library's
  * device code, and so places the array, at that first call: a caller that

@@ -123,7 +123,7 @@ pond_status update_window(pond_ctx* ctx) {
     const int ex = window_extent(sx, dt, 2 * margin) + 5, ey = window_extent(sy, dt, 2 * margin) + 5;
     w.ww = w.tx + ex;
     w.wh = w.ty + ey;
-    w.fx = w.fy = w.fks = w.fww = w.fwh = 0;
+    w.fx = w.fy = w.fks = w.fww = w.fwh = w.wn = w.fwn = 0;
     // cap the staged window at the shared memory a CTA can have; stencils
     // beyond it take the global-memory path
     auto bytes = [](const TileWindow& v) {
@@ -160,7 +160,7 @@ cudaError_t launch_ctx_step_fp64(pond_ctx* ctx, const StateBuf<double>& in,
                                  const StateBuf<double>& out, int32_t* iters, DevStats* stats) {
     if (ctx_staged(ctx))
         return launch_step_staged_fp64(in, out, iters, stats, ctx->grids_dev, ctx->tile_prefix_dev,
-                                       ctx->n_grids, ctx->n_tiles, ctx->N,
+                                       ctx->grids_host[0], ctx->n_grids, ctx->n_tiles, ctx->N,
                                        ctx->n_grids > 1 ? ctx->work_counter : nullptr, ctx->redo,
                                        ctx->win, ctx->persistent_ctas, ctx->L, ctx->P, ctx->stream);
     const GridDesc& G = ctx->grids_host[0];

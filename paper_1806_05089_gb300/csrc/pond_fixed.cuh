@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(TXS* TYS* KS, MINB) k_step_fixed(StagedArgs<do
     static_assert(NT % 32 == 0 && (KS == 1 || KS == 4) && LTX % TXS == 0 && LTY % TYS == 0,
                   "whole warps, the lanes of a node in one");
     extern __shared__ __align__(32) unsigned char smem_raw[];
-    const int WN = A.ww * A.wh;
+    const int WN = A.wn;
     int4* s_h = reinterpret_cast<int4*>(smem_raw);                 // [N1][WN] high words
     int4* s_l = s_h + (size_t)N1 * WN;                             // [N1][WN] low words
     int2* s_gy = reinterpret_cast<int2*>(s_l + (size_t)N1 * WN);   // [Q][NN] y-map of the pass
@@ -349,8 +349,8 @@ __global__ void __launch_bounds__(TXS* TYS* KS, MINB) k_step_fixed(StagedArgs<do
             }
             g = lo;
         }
-        const GridDesc G = A.grids[g];
-        const long long t = tile - A.tile_prefix[g];
+        const GridDesc G = A.n_grids == 1 ? A.grid0 : A.grids[g];
+        const long long t = A.n_grids == 1 ? tile : tile - A.tile_prefix[g];
         const int tiles_x = (G.iw + LTX - 1) / LTX;
         const int ltx0 = G.ix0 + (int)(t % tiles_x) * LTX;
         const int lty0 = G.iy0 + (int)(t / tiles_x) * LTY;
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(TXS* TYS* KS, MINB) k_step_fixed(StagedArgs<do
         const bool fin = isfinite(vxlo) && isfinite(vxhi) && isfinite(vylo) && isfinite(vyhi) &&
                          vxlo > -1.0e6f && vxhi < 1.0e6f && vylo > -1.0e6f && vyhi < 1.0e6f;
         const int ww = fin ? max(1, min(wx1 - wx0 + 1, A.ww)) : 1;
-        const int wh = fin ? max(1, min(wy1 - wy0 + 1, A.wh)) : 1;
+        const int wh = fin ? max(1, min(min(wy1 - wy0 + 1, A.wh), WN / ww)) : 1;
         // (displacements in the fixed-point range of fix_departure)
         in_range = in_range && fin &&
                    fmaxf(fmaxf(fabsf(vxlo), fabsf(vxhi)), fmaxf(fabsf(vylo), fabsf(vyhi))) * fdt < 400.0f;
@@ -748,8 +748,8 @@ __global__ void __launch_bounds__(TXS* TYS* KS, MINB) k_step_fixed(StagedArgs<do
 
 // Dynamic shared memory of k_step_fixed: the staged planes, and per node the
 // y-map and y-weight tables and the stencil tops.
-inline size_t fixed_smem_bytes(int n1, int ww, int wh, int nodes) {
-    return (size_t)n1 * ww * wh * 32 + (size_t)nodes * (8 * (n1 * n1 + 4 * n1) + 4 * n1);
+inline size_t fixed_smem_bytes(int n1, int wn, int nodes) {
+    return (size_t)n1 * wn * 32 + (size_t)nodes * (8 * (n1 * n1 + 4 * n1) + 4 * n1);
 }
 
 }  // namespace pond

@@ -186,7 +186,11 @@ struct TileWindow {
     // per node and staged window
     int fx, fy, fks;
     int fww, fwh;
+    // nodes of the two windows, when they are set by capacity and the sides
+    // only bound a tile's choice (0: ww * wh, fww * fwh)
+    int wn, fwn;
 };
+inline int window_nodes(const TileWindow& w) { return w.wn ? w.wn : w.ww * w.wh; }
 
 // Mixed-precision step over one or many grids (one CTA per tile; batched
 // contexts use a persistent work list).
@@ -205,8 +209,9 @@ cudaError_t launch_step_mixed(const StateBuf<float>& in, const StateBuf<float>& 
 // the first two zero before the first launch (each launch leaves them zero).
 cudaError_t launch_step_staged_fp64(const StateBuf<double>& in, const StateBuf<double>& out,
                                     int32_t* iters, DevStats* stats, const GridDesc* grids_dev,
-                                    const int64_t* tile_prefix_dev, int n_grids, int64_t n_tiles,
-                                    int64_t plane, unsigned int* work_counter, unsigned int* redo,
+                                    const int64_t* tile_prefix_dev, const GridDesc& grid0,
+                                    int n_grids, int64_t n_tiles, int64_t plane,
+                                    unsigned int* work_counter, unsigned int* redo,
                                     const TileWindow& win, int persistent_ctas, const Lattice& L,
                                     const StepParams& P, cudaStream_t s);
 cudaError_t launch_step_staged_mixed(const StateBuf<float>& in, const StateBuf<float>& out,
@@ -234,7 +239,7 @@ inline int window_extent(double span, double dt, double pad) {
 // (as staged_smem_bytes: the FP64 form also holds the y-map table)
 inline size_t staged_window_bytes(const TileWindow& w) {
     const size_t per_node = w.real_bytes == 8 ? 2 : 1;
-    return (size_t)w.n1 * w.ww * w.wh * 4 * w.real_bytes +
+    return (size_t)w.n1 * window_nodes(w) * 4 * w.real_bytes +
            per_node * w.n1 * w.n1 * w.tx * w.ty * w.real_bytes;
 }
 constexpr int STAGED_TY_FP64[2] = {4, 8};

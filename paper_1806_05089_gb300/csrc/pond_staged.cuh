@@ -69,8 +69,9 @@ struct StagedArgs {
     StateBuf<Real> in, out;
     int32_t* iters;
     DevStats* stats;
-    const GridDesc* grids;
+    const GridDesc* grids;        // of a batched context (n_grids > 1)
     const int64_t* tile_prefix;
+    GridDesc grid0;               // the grid of a single-grid launch (FP64 form)
     int n_grids;
     long long n_tiles;
     long long plane;  // plane stride of the packed state
@@ -80,7 +81,7 @@ struct StagedArgs {
     unsigned int* redo_count;
     unsigned int* redo_list;  // entries tile * (sub_x * sub_y) + sub
     int sub_x, sub_y;         // parts of a tile that k_step_fixed's CTAs take
-    int ww, wh;       // allocated window
+    int ww, wh, wn;   // largest window a tile may stage: sides, nodes (FP64 form)
     double c_max;
     float margin;
     StepParams P;
@@ -259,7 +260,7 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
     constexpr unsigned FULL = 0xffffffffu;
     static_assert(TX == 32, "a warp is one tile row");
     extern __shared__ __align__(32) unsigned char smem_raw[];
-    const int WN = A.ww * A.wh;
+    const int WN = Tr::kRedo ? A.wn : A.ww * A.wh;
     Real4* s_f = reinterpret_cast<Real4*>(smem_raw);              // [N1][WN]: row a of g
     Real* s_acc = reinterpret_cast<Real*>(s_f + (size_t)N1 * WN);  // [Q][NT]
     Real* s_ey = s_acc + (size_t)N1 * N1 * NT;  // [Q][NT] Ey[l][b] of the pass (kEyTable)
@@ -310,8 +311,8 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
             }
             g = lo;
         }
-        const GridDesc G = A.grids[g];
-        const long long t = item - A.tile_prefix[g];
+        const GridDesc G = Tr::kRedo && A.n_grids == 1 ? A.grid0 : A.grids[g];
+        const long long t = Tr::kRedo && A.n_grids == 1 ? item : item - A.tile_prefix[g];
         // tiles cover the grid's interior rectangle (the whole grid unless a
         // domain decomposition narrowed it to the part inside its halo)
         const int tiles_x = (G.iw + TX - 1) / TX;
@@ -371,7 +372,7 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
         const bool fin = isfinite(vxlo) && isfinite(vxhi) && isfinite(vylo) && isfinite(vyhi) &&
                          vxlo > -1.0e6f && vxhi < 1.0e6f && vylo > -1.0e6f && vyhi < 1.0e6f;
         const int ww = fin ? max(1, min(wx1 - wx0 + 1, A.ww)) : 1;
-        const int wh = fin ? max(1, min(wy1 - wy0 + 1, A.wh)) : 1;
+        const int wh = fin ? max(1, min(wy1 - wy0 + 1, Tr::kRedo ? min(A.wh, WN / ww) : A.wh)) : 1;
 
         // stage the window, each source re-expressed in lambda_r
         stage_window<Tr, N1>(A.in, A.plane, G, base, wx0, wy0, ww, wh, WN, rux, ruy, rst, s_f,

@@ -742,7 +742,7 @@ static void (*staged64_kernel(int ty, int n1))(StagedArgs<double>) {
 }
 
 static size_t fixed_bytes(const TileWindow& w) {
-    return fixed_smem_bytes(w.n1, w.fww, w.fwh, w.fx * w.fy);
+    return fixed_smem_bytes(w.n1, w.fwn ? w.fwn : w.fww * w.fwh, w.fx * w.fy);
 }
 
 // The attribute is per function and device: only ever raised, so that every
@@ -755,18 +755,8 @@ static cudaError_t raise_smem(void (*kern)(StagedArgs<double>), size_t smem, int
     return e;
 }
 
-cudaError_t staged_prepare_fp64(TileWindow* win, int ex, int ey, int64_t n_tiles, int sms,
-                                int* ctas_per_sm) {
-    static int s_left[64][4] = {{0}}, s_fixed[64][kFixedShapeCount] = {{0}};
-    const int ty = win->ty, n1 = win->n1;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (ty != 4 && ty != 8) return cudaErrorInvalidValue;
-    e = raise_smem(staged64_kernel(ty, n1), staged_window_bytes(*win),
-                   &s_left[dev][(n1 == 3 ? 2 : 0) + (ty == 8 ? 1 : 0)]);
-    if (e != cudaSuccess) return e;
+// The widest part of a tile that suits the number of tiles.
+static int fixed_widest(int n1, int ty, int64_t n_tiles, int sms) {
     // Narrower parts than the whole tile when the tiles do not fill the chip (8
     // wide, four lanes per node; 64^2: 373 -> 131 us a step, 160^2 with 100
     // tiles: 335 -> 321, with 144 tiles slower), or, on D2Q16, where one CTA of
@@ -775,7 +765,33 @@ cudaError_t staged_prepare_fp64(TileWindow* win, int ex, int ey, int64_t n_tiles
     const int64_t waves = (n_tiles + sms - 1) / sms, half_waves = (2 * n_tiles + sms - 1) / sms;
     const bool halves = n1 == 4 && ty == 8 && 53 * half_waves < 100 * waves;
     const int widest = 3 * n_tiles <= 2 * sms ? 8 : halves ? 16 : 32;
-    const size_t cap = 225 * 1024;
+    return widest;
+}
+
+constexpr size_t kFixedSmemCap = 225 * 1024, kStagedSmemCap = 220 * 1024;
+
+// Per-device set-up of the window's two kernels: the resident CTAs per SM of
+// the fixed-point one.
+static cudaError_t fixed_attributes(const TileWindow& win, int pick, int* ctas_per_sm) {
+    static int s_left[64][4] = {{0}}, s_fixed[64][kFixedShapeCount] = {{0}};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    e = raise_smem(staged64_kernel(win.ty, win.n1), staged_window_bytes(win),
+                   &s_left[dev][(win.n1 == 3 ? 2 : 0) + (win.ty == 8 ? 1 : 0)]);
+    if (e != cudaSuccess) return e;
+    const FixedShape& f = kFixedShapes[pick];
+    e = raise_smem(f.kern, fixed_bytes(win), &s_fixed[dev][pick]);
+    if (e != cudaSuccess || !ctas_per_sm) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, f.kern, f.fx * f.fy * f.ks,
+                                                         fixed_bytes(win));
+}
+
+cudaError_t staged_prepare_fp64(TileWindow* win, int ex, int ey, int64_t n_tiles, int sms,
+                                int* ctas_per_sm) {
+    const int ty = win->ty, n1 = win->n1, widest = fixed_widest(n1, ty, n_tiles, sms);
+    if (ty != 4 && ty != 8) return cudaErrorInvalidValue;
     int pick = -1;
     for (int i = 0; i < kFixedShapeCount; ++i) {
         const FixedShape& f = kFixedShapes[i];
@@ -787,23 +803,52 @@ cudaError_t staged_prepare_fp64(TileWindow* win, int ex, int ey, int64_t n_tiles
         win->fks = f.ks;
         win->fww = f.fx + ex;
         win->fwh = f.fy + ey;
-        if (fixed_bytes(*win) <= cap) break;
+        if (fixed_bytes(*win) <= kFixedSmemCap) break;
     }
     if (pick < 0) return cudaErrorInvalidValue;
-    while (fixed_bytes(*win) > cap) {
+    while (fixed_bytes(*win) > kFixedSmemCap) {
         if (win->fww - win->fx >= win->fwh - win->fy) --win->fww; else --win->fwh;
     }
-    const FixedShape& f = kFixedShapes[pick];
-    e = raise_smem(f.kern, fixed_bytes(*win), &s_fixed[dev][pick]);
+    return fixed_attributes(*win, pick, ctas_per_sm);
+}
+
+// The fixed-point launch and the launch over the tiles it leaves (usually
+// none; its CTAs then end at once).
+static cudaError_t launch_fixed(StagedArgs<double> A, const TileWindow& win, int persistent_ctas,
+                                cudaStream_t s) {
+    A.sub_x = win.tx / win.fx;
+    A.sub_y = win.ty / win.fy;
+    A.ww = win.fww;
+    A.wh = win.fwh;
+    A.wn = win.fwn ? win.fwn : win.fww * win.fwh;
+    const FixedShape* f = nullptr;
+    for (const FixedShape& c : kFixedShapes)
+        if (c.n1 == win.n1 && c.ty == win.ty && c.fx == win.fx && c.fy == win.fy && c.ks == win.fks) f = &c;
+    if (!f) return cudaErrorInvalidValue;
+    const int64_t parts = A.n_tiles * A.sub_x * A.sub_y;
+    unsigned int nb = parts > 0 ? (unsigned int)parts : 1u;
+    if (A.work_counter) {
+        cudaError_t e = cudaMemsetAsync(A.work_counter, 0, sizeof(unsigned int), s);
+        if (e != cudaSuccess) return e;
+        if (persistent_ctas < parts) nb = (unsigned int)persistent_ctas;
+    }
+    f->kern<<<nb, f->fx * f->fy * f->ks, fixed_bytes(win), s>>>(A);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, f.kern, f.fx * f.fy * f.ks,
-                                                         fixed_bytes(*win));
+    A.ww = win.ww;
+    A.wh = win.wh;
+    A.wn = window_nodes(win);
+    nb = (unsigned int)(persistent_ctas < A.n_tiles ? persistent_ctas : A.n_tiles);
+    if (nb < 1u) nb = 1u;
+    staged64_kernel(win.ty, win.n1)<<<nb, 32 * win.ty, staged_window_bytes(win), s>>>(A);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_step_staged_fp64(const StateBuf<double>& in, const StateBuf<double>& out,
                                     int32_t* iters, DevStats* stats, const GridDesc* grids_dev,
-                                    const int64_t* tile_prefix_dev, int n_grids, int64_t n_tiles,
-                                    int64_t plane, unsigned int* work_counter, unsigned int* redo,
+                                    const int64_t* tile_prefix_dev, const GridDesc& grid0,
+                                    int n_grids, int64_t n_tiles, int64_t plane,
+                                    unsigned int* work_counter, unsigned int* redo,
                                     const TileWindow& win, int persistent_ctas, const Lattice& L,
                                     const StepParams& P, cudaStream_t s) {
     if (n_tiles == 0) return cudaSuccess;
@@ -815,39 +860,17 @@ cudaError_t launch_step_staged_fp64(const StateBuf<double>& in, const StateBuf<d
     A.stats = stats;
     A.grids = grids_dev;
     A.tile_prefix = tile_prefix_dev;
+    A.grid0 = grid0;
     A.n_grids = n_grids;
     A.n_tiles = n_tiles;
     A.plane = plane;
     A.work_counter = work_counter;
     A.redo_count = redo;
     A.redo_list = redo + 2;
-    A.sub_x = win.tx / win.fx;
-    A.sub_y = win.ty / win.fy;
-    A.ww = win.fww;
-    A.wh = win.fwh;
+    A.P = P;
     A.c_max = L.c_max;
     A.margin = 1.0f;
-    A.P = P;
-    const FixedShape* f = nullptr;
-    for (const FixedShape& c : kFixedShapes)
-        if (c.n1 == L.n1 && c.ty == win.ty && c.fx == win.fx && c.fy == win.fy && c.ks == win.fks) f = &c;
-    if (!f) return cudaErrorInvalidValue;
-    const int64_t parts = n_tiles * A.sub_x * A.sub_y;
-    unsigned int nb = (unsigned int)parts;
-    if (work_counter) {
-        cudaError_t e = cudaMemsetAsync(work_counter, 0, sizeof(unsigned int), s);
-        if (e != cudaSuccess) return e;
-        if (persistent_ctas < parts) nb = (unsigned int)persistent_ctas;
-    }
-    f->kern<<<nb, f->fx * f->fy * f->ks, fixed_bytes(win), s>>>(A);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    // the tiles out of the fixed-point form's range (usually none)
-    A.ww = win.ww;
-    A.wh = win.wh;
-    nb = (unsigned int)(persistent_ctas < n_tiles ? persistent_ctas : n_tiles);
-    staged64_kernel(win.ty, L.n1)<<<nb, 32 * win.ty, staged_window_bytes(win), s>>>(A);
-    return cudaGetLastError();
+    return launch_fixed(A, win, persistent_ctas, s);
 }
 
 }  // namespace pond
@@ -867,6 +890,7 @@ namespace pond {
 
 constexpr int64_t kNoAllocMaxNodes = POND_NOALLOC_MAX_NODES;
 constexpr size_t kNoAllocStatsOffset = 2 * sizeof(double) * (size_t)kNoAllocMaxNodes;
+constexpr size_t kNoAllocRedoOffset = kNoAllocStatsOffset + 192;  // two words
 constexpr size_t kNoAllocBytes = kNoAllocStatsOffset + 256;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
@@ -886,8 +910,8 @@ __global__ void k_noalloc_st_to_t(const double* __restrict__ st, double* __restr
     }
 }
 
-static_assert(sizeof(DevStats) <= 256 && alignof(DevStats) <= 256,
-              "the step counters must fit the 256-byte tail of the scratch array");
+static_assert(sizeof(DevStats) <= 192 && alignof(DevStats) <= 256,
+              "the step counters and two words must fit the 256-byte tail of the scratch array");
 static_assert(kNoAllocStatsOffset % 256 == 0, "the counters' tail must stay 256-byte aligned");
 
 namespace {
@@ -923,12 +947,46 @@ unsigned long long current_context_id() {
 }
 }  // namespace
 
+// The step's kernels for a caller that can neither size the window from the
+// velocities (that would wait for the GPU) nor keep a plan: windows by
+// capacity, each tile taking the sides it needs.
+static TileWindow noalloc_window(int n1, int64_t n_tiles_8, int64_t n_tiles_4, int sms, int* pick) {
+    TileWindow w{};
+    w.tx = 32;
+    w.ty = staged_ty_fp64_default(n1);
+    w.n1 = n1;
+    w.staged = 1;
+    w.real_bytes = 8;
+    const int widest = fixed_widest(n1, w.ty, w.ty == 8 ? n_tiles_8 : n_tiles_4, sms);
+    for (int i = 0; i < kFixedShapeCount; ++i) {
+        const FixedShape& f = kFixedShapes[i];
+        // (no halves: their window, half an SM's, holds T up to about 1.2 T_L)
+        if (f.n1 != n1 || f.ty != w.ty || f.fx == 16 || f.fx > (widest == 16 ? 32 : widest)) continue;
+        *pick = i;
+        w.fx = f.fx;
+        w.fy = f.fy;
+        w.fks = f.ks;
+        break;
+    }
+    // two CTAs per SM for the shapes of two
+    const size_t cap = w.fx * w.fy * w.fks < 256 ? kFixedSmemCap / 2 : kFixedSmemCap;
+    w.fwn = (int)((cap - fixed_smem_bytes(n1, 0, w.fx * w.fy)) / ((size_t)n1 * 32));
+    const size_t tables = 2 * sizeof(double) * n1 * n1 * w.tx * w.ty;
+    w.wn = (int)((kStagedSmemCap - tables) / ((size_t)n1 * 32));
+    w.ww = w.fww = 256;
+    w.wh = w.fwh = 256;
+    return w;
+}
+
 // Every call, with the device current: the device address of the scratch
 // array (its name in host code is only a host-side stand-in; the lookup
 // allocates nothing, but on the first call in a context it may make the
 // driver load this module, which places the array), and, once per context,
 // the lattice constants of this translation unit (a synchronous copy).
-static cudaError_t noalloc_setup(int dev, unsigned char** out) {
+// That first call also launches every kernel the step can pick, over no
+// tiles, so that what the driver sets up at a kernel's first launch (its code
+// and local memory) is in place before the caller reserves device memory.
+static cudaError_t noalloc_setup(int dev, int sms, cudaStream_t s, unsigned char** out) {
     if (dev < 0 || dev >= 256) return cudaErrorInvalidDevice;
     void* p = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
@@ -937,6 +995,19 @@ static cudaError_t noalloc_setup(int dev, unsigned char** out) {
     std::lock_guard<std::mutex> lock(g_noalloc_mu);
     if (id == 0 || g_noalloc_ctx[dev] != id) {
         e = upload_lattice_fp64();
+        if (e != cudaSuccess) return e;
+        StagedArgs<double> none{};
+        none.redo_count = reinterpret_cast<unsigned int*>(static_cast<unsigned char*>(p) + kNoAllocRedoOffset);
+        none.redo_list = none.redo_count;
+        none.n_grids = 1;
+        e = cudaMemsetAsync(none.redo_count, 0, 2 * sizeof(unsigned int), s);
+        for (int n1 = 3; n1 <= 4; ++n1)
+            for (int64_t tiles : {(int64_t)1, (int64_t)sms}) {
+                int pick = -1;
+                const TileWindow w = noalloc_window(n1, tiles, tiles, sms, &pick);
+                if (e == cudaSuccess) e = fixed_attributes(w, pick, nullptr);
+                if (e == cudaSuccess) e = launch_fixed(none, w, 1, s);
+            }
         if (e != cudaSuccess) return e;
         g_noalloc_ctx[dev] = id;
     }
@@ -964,8 +1035,11 @@ extern "C" pond_status pond_step_fp64_noalloc(const pond_config* cfg, int32_t nx
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return POND_ERR_CUDA;
+    int sms = 0;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return POND_ERR_CUDA;
     unsigned char* scratch = nullptr;
-    e = noalloc_setup(dev, &scratch);
+    e = noalloc_setup(dev, sms, static_cast<cudaStream_t>(cuda_stream), &scratch);
     if (e != cudaSuccess) return POND_ERR_CUDA;
 
     const Lattice L = make_lattice(cfg->lattice);
@@ -1000,8 +1074,36 @@ extern "C" pond_status pond_step_fp64_noalloc(const pond_config* cfg, int32_t nx
     out.ux = ux_out;
     out.uy = uy_out;
     out.st = st_out;
-    e = launch_step_fp64(in, out, iters, dstats, nx, ny, L, P,
-                         cfg->nodes_per_warp ? cfg->nodes_per_warp : fp64_default_npw(L.n1), s);
+    if (cfg->nodes_per_warp || cfg->kernel == POND_KERNEL_DIRECT) {
+        e = launch_step_fp64(in, out, iters, dstats, nx, ny, L, P,
+                             cfg->nodes_per_warp ? cfg->nodes_per_warp : fp64_default_npw(L.n1), s);
+    } else {
+        // the staged step, as a context runs it by default (200 x 150: 4.86 ms
+        // with one node per thread of the direct kernel, 0.34 ms so); its list of left-over
+        // tiles goes into T_out, which nothing else touches before the end
+        // (a tile has at least one node, so the list fits)
+        StagedArgs<double> A{};
+        A.in = in;
+        A.out = out;
+        A.iters = iters;
+        A.stats = dstats;
+        A.grid0.nx = A.grid0.iw = nx;
+        A.grid0.ny = A.grid0.ih = ny;
+        A.n_grids = 1;
+        A.plane = N;
+        A.redo_count = reinterpret_cast<unsigned int*>(scratch + kNoAllocRedoOffset);
+        A.redo_list = reinterpret_cast<unsigned int*>(T_out);
+        A.c_max = L.c_max;
+        A.margin = 1.0f;
+        A.P = P;
+        const int64_t tx = (nx + 31) / 32;
+        int pick = -1;
+        const TileWindow w = noalloc_window(L.n1, tx * ((ny + 7) / 8), tx * ((ny + 3) / 4), sms, &pick);
+        A.n_tiles = tx * ((ny + w.ty - 1) / w.ty);
+        e = cudaMemsetAsync(A.redo_count, 0, 2 * sizeof(unsigned int), s);
+        if (e == cudaSuccess) e = fixed_attributes(w, pick, nullptr);
+        if (e == cudaSuccess) e = launch_fixed(A, w, sms, s);
+    }
     if (e != cudaSuccess) return POND_ERR_CUDA;
     k_noalloc_st_to_t<<<nb, 256, 0, s>>>(st_out, T_out, N, L.T_L);
     e = cudaGetLastError();
@@ -1017,7 +1119,7 @@ extern "C" pond_status pond_step_fp64_noalloc(const pond_config* cfg, int32_t nx
         stats->tile_rows = 0;
         stats->nonconverged = (int64_t)h.nonconverged;
         stats->nonphysical = (int64_t)h.nonphysical;
-        stats->halo_fallback = 0;
+        stats->halo_fallback = (int64_t)h.halo_fallback;
         stats->index_faults = (int64_t)h.index_faults;
         if (h.nonphysical) return POND_ERR_NONPHYSICAL;
         if (cfg->strict && h.nonconverged) return POND_ERR_NOT_CONVERGED;

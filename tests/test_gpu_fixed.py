@@ -102,3 +102,28 @@ def test_a_window_too_large_for_whole_tiles_runs_by_halves():
     assert np.abs(a.f - b.f).max() <= TOL64 * np.abs(b.f).max()
     assert np.abs(a.ux - b.ux).max() <= TOL64 * np.sqrt(6.0)
     assert np.max(np.abs(a.T - b.T) / b.T) <= TOL64
+
+
+@pytest.mark.parametrize("lattice", [pond.POND_D2Q16, pond.POND_D2Q9])
+@pytest.mark.parametrize("name,nx,ny", [("plain", 1, 1), ("plain", 37, 1), ("plain", 1, 70),
+                                        ("plain", 500, 90), ("density", 160, 12), ("shear", 300, 96)])
+def test_allocation_free_step_matches_the_context_step(name, nx, ny, lattice):
+    """Windows sized by capacity against windows sized by the velocities: the
+    same staged values and sums, so bit for bit."""
+    import torch
+    T_L = 1.0 / 3.0 if lattice == pond.POND_D2Q9 else 1.0
+    fields = field(name, nx, ny, T_L)
+    cfg = pond.pond_config_default(pond.POND_FP64)
+    cfg.lattice, cfg.T_ref = lattice, T_L
+    with pond.Sim(nx, ny, pond.POND_FP64, lattice=lattice, T_ref=T_L) as s:
+        s.set_state(fields.rho, fields.ux, fields.uy, fields.T)
+        start = s.state()
+        s.set_state(None, start.ux, start.uy, start.T, start.f)
+        s.step(1)
+        want = s.state()
+    cur = [torch.tensor(a, device="cuda") for a in (start.f, start.ux, start.uy, start.T)]
+    out = [torch.empty_like(a) for a in cur]
+    stats = pond.pond_step_fp64_noalloc(cfg, *cur, *out)
+    assert stats["nonphysical"] == 0 and stats["halo_fallback"] == 0
+    for a, b in zip(out, (want.f, want.ux, want.uy, want.T)):
+        assert np.array_equal(a.cpu().numpy(), b)
