@@ -109,6 +109,14 @@ __device__ __forceinline__ int wrap_idx(long long v, int n) {
     return (int)(r < 0 ? r + n : r);
 }
 
+// Periodic wrap of an index that is mostly within one period of the grid: a
+// few instructions there, the 64-bit remainder (a hundred) beyond.
+__device__ __forceinline__ int wrap_near(int v, int n) {
+    v = v < 0 ? v + n : v;
+    v = v >= n ? v - n : v;
+    return (unsigned)v < (unsigned)n ? v : wrap_idx((long long)v, n);
+}
+
 // Index + small offset (0..3) wrapped, for an already wrapped base.
 __device__ __forceinline__ int wrap_inc(int base, int off, int n) {
     int v = base + off;

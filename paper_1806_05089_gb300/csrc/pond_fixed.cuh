@@ -194,10 +194,11 @@ __device__ __forceinline__ bool stage_window_fixed(const StateBuf<double>& in, l
     const double inv_rst = kFixOne / rst;
     bool ok = true;
     (void)stats;
+    const float inv_ww = 1.0f / (float)ww;
     for (int i = tid; i < ww * wh; i += nt) {
-        const int cx = i % ww, cy = i / ww;
-        const int gx = wrap_idx((long long)wx0 + cx, G.nx);
-        const int gy = wrap_idx((long long)wy0 + cy, G.ny);
+        const int cy = window_row(i, inv_ww), cx = i - cy * ww;
+        const int gx = wrap_near(wx0 + cx, G.nx);
+        const int gy = wrap_near(wy0 + cy, G.ny);
         const long long gi = base + (long long)gy * G.nx + gx;
         if (!POND_INDEX_OK(gx >= 0 && gx < G.nx && gy >= 0 && gy < G.ny && i < WN, stats))
             continue;

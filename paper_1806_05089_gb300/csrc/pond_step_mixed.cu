@@ -121,11 +121,14 @@ __device__ __noinline__ float stencil_global(const MixedArgs& A, const GridDesc&
 // the Taylor offsets of that transform: xi_a = c_a + c_a r + d.  Kept out of
 // line so the pass loop keeps its register budget.
 template <int N1, class Args>
-__device__ __noinline__ void finish_node(const Args& A, float* s_acc, int NT, int tid,
+__device__ __noinline__ void finish_node(const Args& A, const float* s_acc, int NT, int tid,
                                          long long node, bool regauge, float r, float dx,
                                          float dy, double ux, double uy, double st, float rho) {
     constexpr int Q = N1 * N1;
     const LatticeF& L = c_Lf[lattice_slot(N1)];
+    float f[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) f[q] = s_acc[q * NT + tid];
     if (regauge) {
         // In correction form, f + (G - I) f: at convergence G - I is of the
         // size of the last gauge increment (~1e-7 to 1e-6), so writing the
@@ -144,9 +147,7 @@ __device__ __noinline__ void finish_node(const Args& A, float* s_acc, int NT, in
                 ey[k][a] = gauge_tail<N1>(L.d3[k], L.d2[k][a], L.d1[k][a], dey) * dey;
             }
         }
-        float f[Q], H[Q];
-#pragma unroll
-        for (int q = 0; q < Q; ++q) f[q] = s_acc[q * NT + tid];
+        float H[Q], o[Q];
 #pragma unroll
         for (int a = 0; a < N1; ++a)
 #pragma unroll
@@ -163,8 +164,10 @@ __device__ __noinline__ void finish_node(const Args& A, float* s_acc, int NT, in
                 float c = H[N1 * k + l];
 #pragma unroll
                 for (int a = 0; a < N1; ++a) c = fmaf(ex[k][a], f[N1 * a + l] + H[N1 * a + l], c);
-                s_acc[(N1 * k + l) * NT + tid] = f[N1 * k + l] + c;
+                o[N1 * k + l] = f[N1 * k + l] + c;
             }
+#pragma unroll
+        for (int q = 0; q < Q; ++q) f[q] = o[q];
     }
     // BGK in FP32, kept exactly conservative: the relaxed non-equilibrium
     // part n = f - rho W is first stripped of its mass, momentum and energy
@@ -183,7 +186,7 @@ __device__ __noinline__ void finish_node(const Args& A, float* s_acc, int NT, in
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
         const int k = q / N1, l = q % N1;
-        const float n = fmaf(-rho, L.w[k] * L.w[l], s_acc[q * NT + tid]);
+        const float n = fmaf(-rho, L.w[k] * L.w[l], f[q]);
         M0 += n;
         M1 = fmaf(L.c[k], n, M1);
         M2 = fmaf(L.c[l], n, M2);
@@ -203,7 +206,7 @@ __device__ __noinline__ void finish_node(const Args& A, float* s_acc, int NT, in
         const int k = q / N1, l = q % N1;
         const float Wq = L.w[k] * L.w[l];
         const float c2 = fmaf(L.c[k], L.c[k], L.c[l] * L.c[l]);
-        const float a = s_acc[q * NT + tid];
+        const float a = f[q];
         float n = fmaf(-rho, Wq, a);
         const float proj = fmaf(M0, fmaf(e2, c2, e0),
                                 fmaf(M1, L.c[k], fmaf(M2, L.c[l], M3 * fmaf(t2, c2, t0))));
