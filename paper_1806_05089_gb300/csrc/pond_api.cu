@@ -414,7 +414,7 @@ pond_status pond_create(const pond_config* cfg, int32_t n_grids, const int32_t* 
     ok = ok && alloc((void**)&ctx->grids_dev, sizeof(GridDesc) * n_grids, "alloc grids");
     ok = ok && alloc((void**)&ctx->tile_prefix_dev, sizeof(int64_t) * (n_grids + 1), "alloc prefix");
     ok = ok && alloc((void**)&ctx->work_counter, sizeof(unsigned int), "alloc counter");
-    ok = ok && alloc((void**)&ctx->bounds_dev, 8 * sizeof(float), "alloc bounds");
+    ok = ok && alloc((void**)&ctx->bounds_dev, 8 * sizeof(unsigned int), "alloc bounds");
     size_t redo_words = 0;
     if (!mixed(ctx) && ctx_staged(ctx)) {
         // two counters and the 8-node-wide parts of the finest FP64 tiles
@@ -531,26 +531,23 @@ pond_status pond_set_state(pond_ctx* ctx, int32_t grid, const void* rho, const v
     }
     if (mixed(ctx)) {
         CK(launch_init_state<float>(d_rho, d_ux, d_uy, d_T, d_f, buf<float>(ctx, ctx->cur, G.offset),
-                                    n, ctx->N, ctx->L, ctx->stream),
+                                    n, ctx->N, ctx->L, ctx->bounds_dev, ctx->stream),
            "init state");
     } else {
         CK(launch_init_state<double>(d_rho, d_ux, d_uy, d_T, d_f,
                                      buf<double>(ctx, ctx->cur, G.offset), n, ctx->N, ctx->L,
-                                     ctx->stream),
+                                     ctx->bounds_dev, ctx->stream),
            "init state");
     }
-    // velocity spans of this grid, for the tile kernels' windows, and the
-    // count of nodes with T <= 0 or a non-finite gauge (the gauge is checked
+    // with the velocity spans of this grid, for the tile kernels' windows, and
+    // the count of nodes with T <= 0 or a non-finite gauge (the gauge is checked
     // on the device, in the same pass, for host and device input alike)
-    CK(launch_disp_bounds(ctx->ux[ctx->cur] + G.offset, ctx->uy[ctx->cur] + G.offset,
-                          ctx->st[ctx->cur] + G.offset, n, ctx->L.c_max, ctx->bounds_dev,
-                          ctx->stream),
-       "bounds");
-    float b5[5];
-    CK(cudaMemcpyAsync(b5, ctx->bounds_dev, sizeof b5, cudaMemcpyDeviceToHost, ctx->stream), "D2H bounds");
+    unsigned int enc[5];
+    CK(cudaMemcpyAsync(enc, ctx->bounds_dev, sizeof enc, cudaMemcpyDeviceToHost, ctx->stream), "D2H bounds");
     CK(cudaStreamSynchronize(ctx->stream), "set_state sync");
+    float b5[4];
     unsigned int bad = 0;
-    std::memcpy(&bad, &b5[4], sizeof bad);
+    decode_bounds(enc, b5, &bad);
     if (bad != 0 || !(std::isfinite(b5[0]) && std::isfinite(b5[1]) && std::isfinite(b5[2]) &&
                       std::isfinite(b5[3]))) {
         // the grid's buffers now hold the refused state: no step runs on it
@@ -850,10 +847,13 @@ pond_status pond_max_displacement(pond_ctx* ctx, int32_t grid, double* out) {
                           ctx->st[ctx->cur] + G.offset, n, ctx->L.c_max, ctx->bounds_dev,
                           ctx->stream),
        "bounds");
-    float b4[4];
-    CK(cudaMemcpyAsync(b4, ctx->bounds_dev, sizeof b4, cudaMemcpyDeviceToHost, ctx->stream),
+    unsigned int enc[5];
+    CK(cudaMemcpyAsync(enc, ctx->bounds_dev, sizeof enc, cudaMemcpyDeviceToHost, ctx->stream),
        "D2H bounds");
     CK(cudaStreamSynchronize(ctx->stream), "bounds sync");
+    float b4[4];
+    unsigned int bad = 0;
+    decode_bounds(enc, b4, &bad);
     double m = 0.0;
     for (int i = 0; i < 4; ++i) m = std::fmax(m, std::fabs((double)b4[i]));
     *out = m * ctx->cfg.dt;

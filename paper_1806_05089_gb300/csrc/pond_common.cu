@@ -1,6 +1,7 @@
 // pond_common.cu -- lattice constants, state initialisation / read-out and
 // displacement bounds for the PonD library.
 #include <cmath>
+#include <cstring>
 
 #include "pond_device.cuh"
 
@@ -87,107 +88,51 @@ LatticeF to_float(const Lattice& L) {
     return F;
 }
 
-// f_q = rho W_q in the node's own gauge (Eq. equilibrium), or a copy of the
-// given FP64 populations; T -> sqrt(theta).
-template <typename Real>
-__global__ void k_init_state(const double* __restrict__ rho, const double* __restrict__ ux,
-                             const double* __restrict__ uy, const double* __restrict__ T,
-                             const double* __restrict__ f_given, StateBuf<Real> st, int64_t N,
-                             int64_t plane, Lattice L) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    st.ux[i] = ux[i];
-    st.uy[i] = uy[i];
-    st.st[i] = sqrt(T[i] / L.T_L);
-    if (f_given) {
-        for (int q = 0; q < L.q; ++q) st.f[q * plane + i] = (Real)f_given[q * N + i];
-    } else {
-        const double r = rho[i];
-        for (int q = 0; q < L.q; ++q)
-            st.f[q * plane + i] = (Real)(r * L.w[q / L.n1] * L.w[q % L.n1]);
-    }
+// FP64 <-> FP32 on the integer pipe.  The conversion instructions share the
+// FP64 pipe (2 a clock and SM), which held the state I/O below at a third of
+// the memory rate.  Exact; to FP32 rounded to nearest even.  Zeros, FP32
+// subnormals, infinities and NaN take the instruction.
+__device__ __forceinline__ double widen(float v) {
+    const unsigned int b = __float_as_uint(v);
+    if ((b & 0x7f800000u) - 0x00800000u >= 0x7f000000u) return (double)v;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))),
+                            (int)(b << 29));
 }
 
+__device__ __forceinline__ float narrow(double v) {
+    const unsigned int hi = (unsigned int)__double2hiint(v), lo = (unsigned int)__double2loint(v);
+    const unsigned int e = hi >> 20 & 0x7ffu;
+    if (e - 897u >= 253u) return (float)v;
+    const unsigned int m = (e - 896u) << 23 | (hi & 0xfffffu) << 3 | lo >> 29;
+    // the first bit below, and a tie to even
+    const unsigned int up = (lo >> 28 & 1u) & (((lo & 0x0fffffffu) | (m & 1u)) != 0u ? 1u : 0u);
+    return __uint_as_float((hi & 0x80000000u) | (m + up));
+}
+__device__ __forceinline__ double widen(double v) { return v; }
 template <typename Real>
-cudaError_t launch_init_state(const double* rho, const double* ux, const double* uy,
-                              const double* T, const double* f_given, StateBuf<Real> st,
-                              int64_t N, int64_t plane, const Lattice& L, cudaStream_t s) {
-    if (N == 0) return cudaSuccess;
-    const int bs = 256;
-    const unsigned nb = (unsigned)((N + bs - 1) / bs);
-    k_init_state<Real><<<nb, bs, 0, s>>>(rho, ux, uy, T, f_given, st, N, plane, L);
-    return cudaGetLastError();
+__device__ __forceinline__ Real narrow_to(double v) {
+    if constexpr (sizeof(Real) == 4) return narrow(v);
+    else return v;
 }
 
-template <typename Real>
-__global__ void k_read_state(StateBuf<Real> st, int64_t N, int64_t plane, double* rho,
-                             double* ux, double* uy, double* T, double* f, Lattice L) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    double r = 0.0;
-    for (int q = 0; q < L.q; ++q) {
-        const double v = (double)st.f[q * plane + i];
-        r += v;
-        if (f) f[q * N + i] = v;
-    }
-    if (rho) rho[i] = r;
-    if (ux) ux[i] = st.ux[i];
-    if (uy) uy[i] = st.uy[i];
-    if (T) {
-        const double s = st.st[i];
-        T[i] = s * s * L.T_L;
-    }
+__device__ __forceinline__ bool finite_bits(double v) {
+    return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000;
 }
 
-template <typename Real>
-cudaError_t launch_read_state(StateBuf<Real> st, int64_t N, int64_t plane, double* rho,
-                              double* ux, double* uy, double* T, double* f, const Lattice& L,
-                              cudaStream_t s) {
-    if (N == 0) return cudaSuccess;
-    const int bs = 256;
-    const unsigned nb = (unsigned)((N + bs - 1) / bs);
-    k_read_state<Real><<<nb, bs, 0, s>>>(st, N, plane, rho, ux, uy, T, f, L);
-    return cudaGetLastError();
-}
-
-template cudaError_t launch_init_state<double>(const double*, const double*, const double*,
-                                               const double*, const double*, StateBuf<double>,
-                                               int64_t, int64_t, const Lattice&, cudaStream_t);
-template cudaError_t launch_init_state<float>(const double*, const double*, const double*,
-                                              const double*, const double*, StateBuf<float>,
-                                              int64_t, int64_t, const Lattice&, cudaStream_t);
-template cudaError_t launch_read_state<double>(StateBuf<double>, int64_t, int64_t, double*,
-                                               double*, double*, double*, double*,
-                                               const Lattice&, cudaStream_t);
-template cudaError_t launch_read_state<float>(StateBuf<float>, int64_t, int64_t, double*,
-                                              double*, double*, double*, double*,
-                                              const Lattice&, cudaStream_t);
-
-// Bounds of the particle velocities over a grid: out4 = {min(u_x - c_max st),
-// max(u_x + c_max st), min(u_y - c_max st), max(u_y + c_max st)} (as floats,
-// combined by integer atomics on an order-preserving encoding).
+// Order-preserving encoding of a float, larger for a larger value; never 0 for
+// a number, so that a zeroed word is below all.
 __device__ __forceinline__ unsigned int f2ord(float f) {
     const unsigned int u = __float_as_uint(f);
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-__global__ void k_disp_bounds(const double* __restrict__ ux, const double* __restrict__ uy,
-                              const double* __restrict__ st, int64_t N, double cmax,
-                              unsigned int* out5) {
-    float lo_x = 3.0e38f, hi_x = -3.0e38f, lo_y = 3.0e38f, hi_y = -3.0e38f;
-    unsigned int bad = 0u;  // nodes with s <= 0 or a non-finite gauge
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const double x = ux[i], y = uy[i], t = st[i];
-        bad += (t > 0.0 && isfinite(t) && isfinite(x) && isfinite(y)) ? 0u : 1u;
-        const double s = cmax * t;
-        lo_x = fminf(lo_x, (float)(x - s));
-        hi_x = fmaxf(hi_x, (float)(x + s));
-        lo_y = fminf(lo_y, (float)(y - s));
-        hi_y = fmaxf(hi_y, (float)(y + s));
-    }
-    // warp, then block reduction: one atomic per block and value (atomics on
-    // one address serialise, so one per warp would dominate the pass)
+// Block reduction of the particle-velocity bounds {min x, max x, min y, max y}
+// and of the count of bad nodes into out5: the maxima encoded by f2ord, the
+// minima as the complement of it (all five words start at zero; decode_bounds
+// reads them).  Warp, then block: one atomic per block and value, as atomics on
+// one address serialise.  All threads of the block take part.
+__device__ __forceinline__ void reduce_bounds(float lo_x, float hi_x, float lo_y, float hi_y,
+                                              unsigned int bad, unsigned int* out5) {
     __shared__ float s_b[4][32];
     __shared__ unsigned int s_bad[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -217,27 +162,164 @@ __global__ void k_disp_bounds(const double* __restrict__ ux, const double* __res
         bad = in ? s_bad[lane] : 0u;
     }
     if (lane == 0) {
-        atomicMin(out5 + 0, f2ord(lo_x));
+        atomicMax(out5 + 0, ~f2ord(lo_x));
         atomicMax(out5 + 1, f2ord(hi_x));
-        atomicMin(out5 + 2, f2ord(lo_y));
+        atomicMax(out5 + 2, ~f2ord(lo_y));
         atomicMax(out5 + 3, f2ord(hi_y));
         if (bad) atomicAdd(out5 + 4, bad);
     }
 }
 
-__global__ void k_ord_to_float(unsigned int* v) {
-    const int i = threadIdx.x;
-    if (i < 4) {
-        const unsigned int u = v[i];
+void decode_bounds(const unsigned int in5[5], float out4[4], unsigned int* bad) {
+    for (int i = 0; i < 4; ++i) {
+        const unsigned int u = (i & 1) ? in5[i] : ~in5[i];
         const unsigned int b = (u & 0x80000000u) ? (u & 0x7fffffffu) : ~u;
-        v[i] = b;  // now the float bit pattern
+        std::memcpy(&out4[i], &b, sizeof b);
+    }
+    *bad = in5[4];
+}
+
+// f_q = rho W_q in the node's own gauge (Eq. equilibrium), or a copy of the
+// given FP64 populations; T -> sqrt(theta).  The same pass bounds the particle
+// velocities (in FP32: they size the staged windows, which have a node of
+// margin) and counts the nodes with T <= 0 or a non-finite gauge, into out5.
+// Of FP64 arithmetic a node needs the root, 2 + 4 products (the weights take two
+// values per dimension) and, on D2Q9, the division by T_L: 2048^2 mixed, with
+// the former pass for the bounds, 597 -> 185 us.
+template <typename Real, int N1>
+__global__ void __launch_bounds__(256)
+k_init_state(const double* __restrict__ rho, const double* __restrict__ ux,
+             const double* __restrict__ uy, const double* __restrict__ T,
+             const double* __restrict__ f_given, StateBuf<Real> st, int64_t N, int64_t plane,
+             Lattice L, unsigned int* __restrict__ out5) {
+    constexpr int Q = N1 * N1;
+    float lo_x = 3.0e38f, hi_x = -3.0e38f, lo_y = 3.0e38f, hi_y = -3.0e38f;
+    unsigned int bad = 0u;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < N) {
+        const double x = ux[i], y = uy[i];
+        const double t = sqrt(N1 == 4 ? T[i] : T[i] / L.T_L);  // T_L = 1 on D2Q16
+        st.ux[i] = x;
+        st.uy[i] = y;
+        st.st[i] = t;
+        if (f_given) {
+#pragma unroll
+            for (int q = 0; q < Q; ++q) st.f[q * plane + i] = narrow_to<Real>(f_given[q * N + i]);
+        } else {
+            // populations (k, l) by the classes of k and l: inner, outer speed
+            const double r = rho[i], ri = r * L.w[1], ro = r * L.w[0];
+            const Real ii = narrow_to<Real>(ri * L.w[1]), io = narrow_to<Real>(ri * L.w[0]);
+            const Real oi = narrow_to<Real>(ro * L.w[1]), oo = narrow_to<Real>(ro * L.w[0]);
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const bool ko = q / N1 == 0 || q / N1 == N1 - 1, lo = q % N1 == 0 || q % N1 == N1 - 1;
+                st.f[q * plane + i] = ko ? (lo ? oo : oi) : (lo ? io : ii);
+            }
+        }
+        bad = __double2hiint(t) >= 0 && t != 0.0 && finite_bits(t) && finite_bits(x) && finite_bits(y) ? 0u : 1u;
+        const float xf = narrow(x), yf = narrow(y), s = (float)L.c_max * narrow(t);
+        lo_x = xf - s;
+        hi_x = xf + s;
+        lo_y = yf - s;
+        hi_y = yf + s;
+    }
+    reduce_bounds(lo_x, hi_x, lo_y, hi_y, bad, out5);
+}
+
+template <typename Real>
+cudaError_t launch_init_state(const double* rho, const double* ux, const double* uy,
+                              const double* T, const double* f_given, StateBuf<Real> st,
+                              int64_t N, int64_t plane, const Lattice& L, unsigned int* out5,
+                              cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(out5, 0, 5 * sizeof(unsigned int), s);
+    if (e != cudaSuccess || N == 0) return e;
+    const int bs = 256;
+    const unsigned nb = (unsigned)((N + bs - 1) / bs);
+    if (L.n1 == 4)
+        k_init_state<Real, 4><<<nb, bs, 0, s>>>(rho, ux, uy, T, f_given, st, N, plane, L, out5);
+    else
+        k_init_state<Real, 3><<<nb, bs, 0, s>>>(rho, ux, uy, T, f_given, st, N, plane, L, out5);
+    return cudaGetLastError();
+}
+
+// Bound by memory: the density's sum (16 dependent FP64 additions) is formed
+// only where it is asked for, and FP32 populations are widened on the integer
+// pipe.  2048^2 mixed, populations and gauge: 271 -> 148 us (6.8 TB/s).
+template <typename Real, int N1, bool RHO>
+__global__ void __launch_bounds__(256)
+k_read_state(StateBuf<Real> st, int64_t N, int64_t plane, double* __restrict__ rho,
+             double* __restrict__ ux, double* __restrict__ uy, double* __restrict__ T,
+             double* __restrict__ f, double T_L) {
+    constexpr int Q = N1 * N1;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    if (RHO || f) {
+        double r = 0.0;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const double v = widen(st.f[q * plane + i]);
+            if (RHO) r += v;
+            if (f) f[q * N + i] = v;
+        }
+        if (RHO) rho[i] = r;
+    }
+    if (ux) ux[i] = st.ux[i];
+    if (uy) uy[i] = st.uy[i];
+    if (T) {
+        const double s = st.st[i];
+        T[i] = s * s * T_L;
     }
 }
 
-__global__ void k_bounds_reset(unsigned int* v) {
-    const int i = threadIdx.x;
-    if (i < 4) v[i] = (i & 1) ? 0u : 0xffffffffu;
-    if (i == 4) v[4] = 0u;
+template <typename Real>
+cudaError_t launch_read_state(StateBuf<Real> st, int64_t N, int64_t plane, double* rho,
+                              double* ux, double* uy, double* T, double* f, const Lattice& L,
+                              cudaStream_t s) {
+    if (N == 0) return cudaSuccess;
+    const int bs = 256;
+    const unsigned nb = (unsigned)((N + bs - 1) / bs);
+    if (L.n1 == 4) {
+        if (rho) k_read_state<Real, 4, true><<<nb, bs, 0, s>>>(st, N, plane, rho, ux, uy, T, f, L.T_L);
+        else k_read_state<Real, 4, false><<<nb, bs, 0, s>>>(st, N, plane, rho, ux, uy, T, f, L.T_L);
+    } else {
+        if (rho) k_read_state<Real, 3, true><<<nb, bs, 0, s>>>(st, N, plane, rho, ux, uy, T, f, L.T_L);
+        else k_read_state<Real, 3, false><<<nb, bs, 0, s>>>(st, N, plane, rho, ux, uy, T, f, L.T_L);
+    }
+    return cudaGetLastError();
+}
+
+template cudaError_t launch_init_state<double>(const double*, const double*, const double*,
+                                               const double*, const double*, StateBuf<double>,
+                                               int64_t, int64_t, const Lattice&, unsigned int*,
+                                               cudaStream_t);
+template cudaError_t launch_init_state<float>(const double*, const double*, const double*,
+                                              const double*, const double*, StateBuf<float>,
+                                              int64_t, int64_t, const Lattice&, unsigned int*,
+                                              cudaStream_t);
+template cudaError_t launch_read_state<double>(StateBuf<double>, int64_t, int64_t, double*,
+                                               double*, double*, double*, double*,
+                                               const Lattice&, cudaStream_t);
+template cudaError_t launch_read_state<float>(StateBuf<float>, int64_t, int64_t, double*,
+                                              double*, double*, double*, double*,
+                                              const Lattice&, cudaStream_t);
+
+// Bounds of the particle velocities over a grid, from the FP64 values.
+__global__ void k_disp_bounds(const double* __restrict__ ux, const double* __restrict__ uy,
+                              const double* __restrict__ st, int64_t N, double cmax,
+                              unsigned int* out5) {
+    float lo_x = 3.0e38f, hi_x = -3.0e38f, lo_y = 3.0e38f, hi_y = -3.0e38f;
+    unsigned int bad = 0u;  // nodes with s <= 0 or a non-finite gauge
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const double x = ux[i], y = uy[i], t = st[i];
+        bad += (t > 0.0 && isfinite(t) && isfinite(x) && isfinite(y)) ? 0u : 1u;
+        const double s = cmax * t;
+        lo_x = fminf(lo_x, (float)(x - s));
+        hi_x = fmaxf(hi_x, (float)(x + s));
+        lo_y = fminf(lo_y, (float)(y - s));
+        hi_y = fmaxf(hi_y, (float)(y + s));
+    }
+    reduce_bounds(lo_x, hi_x, lo_y, hi_y, bad, out5);
 }
 
 // Halo strips of a domain decomposition: a rectangle of the state to or from
@@ -298,15 +380,14 @@ template cudaError_t launch_unpack_rect<float>(StateBuf<float>, int, int, int, i
                                                int64_t, const double*, cudaStream_t);
 
 cudaError_t launch_disp_bounds(const double* ux, const double* uy, const double* st, int64_t N,
-                               double c_max, float* out5, cudaStream_t s) {
-    unsigned int* o = reinterpret_cast<unsigned int*>(out5);
-    k_bounds_reset<<<1, 32, 0, s>>>(o);
+                               double c_max, unsigned int* out5, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(out5, 0, 5 * sizeof(unsigned int), s);
+    if (e != cudaSuccess) return e;
     const int bs = 256;
     int64_t nb = (N + bs - 1) / bs;
     if (nb > 256) nb = 256;
     if (nb < 1) nb = 1;
-    k_disp_bounds<<<(unsigned)nb, bs, 0, s>>>(ux, uy, st, N, c_max, o);
-    k_ord_to_float<<<1, 32, 0, s>>>(o);
+    k_disp_bounds<<<(unsigned)nb, bs, 0, s>>>(ux, uy, st, N, c_max, out5);
     return cudaGetLastError();
 }
 

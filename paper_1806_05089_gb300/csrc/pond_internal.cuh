@@ -258,11 +258,14 @@ constexpr int MIXED_TY_CHOICES[4] = {4, 8, 16, -16};
 size_t mixed_smem_bytes(const TileWindow& w);
 cudaError_t mixed_prepare(int ty, bool pair, int n1, size_t smem_bytes, int* ctas_per_sm);
 
-// Equilibrium initialisation f = rho W (Eq. equilibrium) and T -> sqrt(theta).
+// Equilibrium initialisation f = rho W (Eq. equilibrium) and T -> sqrt(theta);
+// out5 gets the bounds of the particle velocities and the count of nodes with
+// T <= 0 or a non-finite gauge, encoded (decode_bounds).
 template <typename Real>
 cudaError_t launch_init_state(const double* rho, const double* ux, const double* uy,
                               const double* T, const double* f_given, StateBuf<Real> st,
-                              int64_t N, int64_t plane, const Lattice& L, cudaStream_t s);
+                              int64_t N, int64_t plane, const Lattice& L, unsigned int* out5,
+                              cudaStream_t s);
 
 // rho = sum f, T = st^2 T_L, and f (as FP64) read-out.
 template <typename Real>
@@ -282,10 +285,11 @@ cudaError_t launch_unpack_rect(StateBuf<Real> st, int nx, int x0, int y0, int w,
 
 // Bounds of the particle velocities over the nodes, {min (u_x - c_max st),
 // max (u_x + c_max st), min (u_y - c_max st), max (u_y + c_max st)} as
-// floats in out5[0..3], and in out5[4] (read as an unsigned int) the number
-// of nodes with st <= 0 or a non-finite gauge.
+// floats, and the number of nodes with st <= 0 or a non-finite gauge, encoded in
+// out5; decode_bounds reads a host copy of it.
 cudaError_t launch_disp_bounds(const double* ux, const double* uy, const double* st,
-                               int64_t N, double c_max, float* out5, cudaStream_t s);
+                               int64_t N, double c_max, unsigned int* out5, cudaStream_t s);
+void decode_bounds(const unsigned int in5[5], float out4[4], unsigned int* bad);
 
 // Adjoint (pond_adjoint.cu, pond_adjoint_mixed.cu).
 struct AdjointScratch;
@@ -320,7 +324,7 @@ struct pond_ctx {
     int64_t* tile_prefix_dev = nullptr;
     unsigned int* work_counter = nullptr;
     unsigned int* redo = nullptr;  // staged FP64 step: tiles left to the FP64 kernel
-    float* bounds_dev = nullptr;
+    unsigned int* bounds_dev = nullptr;  // encoded velocity bounds (decode_bounds)
     int64_t n_tiles = 0;
     int tile_ty = pond::MIXED_TY;  // rows of the mixed kernel's tile
     bool tile_pair = false;        // paired kernel (two stacked nodes per thread)
