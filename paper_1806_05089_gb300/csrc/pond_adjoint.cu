@@ -35,16 +35,20 @@
 #include <cmath>
 
 #include "pond_device.cuh"
-#include "pond_staged.cuh"
+#include "pond_fixed.cuh"
 
 namespace pond {
 
 // Lattice constants of the adjoint kernels, slot lattice_slot(n1).
 __constant__ Lattice c_La[2];
+__constant__ LatticeFix c_Lafix[2];
 
 cudaError_t upload_lattice_adjoint() {
     const Lattice L[2] = {make_lattice(POND_D2Q16), make_lattice(POND_D2Q9)};
-    return cudaMemcpyToSymbol(c_La, L, sizeof(L));
+    const LatticeFix F[2] = {make_lattice_fix(L[0]), make_lattice_fix(L[1])};
+    cudaError_t e = cudaMemcpyToSymbol(c_La, L, sizeof(L));
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_Lafix, F, sizeof(F));
+    return e;
 }
 
 struct AdjointScratch {
@@ -57,6 +61,10 @@ struct AdjointScratch {
     double* minmax = nullptr;    // 6 doubles: min/max of ux*, uy*, s*
     int2* org = nullptr;         // [16][N] stencil origin of (q, t), relative to t
     double* lw = nullptr;        // [16][N][8] cubic weights of (q, t): x 0..3, y 0..3
+    // staged contexts keep org and lw per speed and direction instead
+    int* org1 = nullptr;         // [2][4][N]
+    double* lw1 = nullptr;       // [2][4][N][4]
+    unsigned int* redo = nullptr;  // phase A: {count, tiles, marks} left to the FP64 kernel
     double* inv_st = nullptr;    // [N] 1 / s* at every target
     double* jvp = nullptr;       // [4][16][N] A*, dA/du_x, dA/du_y, dA/ds (staged phase A)
     double* nu_dev = nullptr;    // nu cotangent of calls with nu_bar_accum == NULL
@@ -97,8 +105,11 @@ struct AdjArgs {
     double* beta_bar;
     // per (population, target), written by the target kernel for the gather:
     // stencil origin relative to the target, cubic weights, and 1 / s*
+    // (staged contexts: per speed and direction)
     int2* org;
     double* lw;
+    int *org_x, *org_y;      // [n1][N]
+    double *lw_x, *lw_y;     // [n1][N][4]
     double* inv_st;
     int nx, ny;
     long long N;
@@ -466,8 +477,8 @@ __global__ void __launch_bounds__(ADJ_GATHER_WARPS * 32) k_adjoint_sources_t(Adj
             const long long t = (long long)wrap_idx(yy, A.ny) * A.nx + wrap_idx(xx, A.nx);
 #pragma unroll
             for (int i = 0; i < N1; ++i) {
-                const int jx = JX - (xx + A.org[(long long)(N1 * i) * A.N + t].x);
-                const int jy = JY - (yy + A.org[(long long)i * A.N + t].y);
+                const int jx = JX - (xx + A.org_x[(long long)i * A.N + t]);
+                const int jy = JY - (yy + A.org_y[(long long)i * A.N + t]);
                 my.jx[i] = (signed char)jx;
                 my.jy[i] = (signed char)jy;
                 kmask |= (jx >= 0 && jx <= 3) ? 1u << i : 0u;
@@ -522,11 +533,11 @@ __global__ void __launch_bounds__(ADJ_GATHER_WARPS * 32) k_adjoint_sources_t(Adj
                 row[a] = gauge_poly<N1>(L.d3[i], L.d2[i][a], L.d1[i][a], a == i ? 1.0 : 0.0,
                                         fma(L.c[a], r, base));
             if (yrow) {
-                g.ly[i] = A.lw[8 * ((long long)i * A.N + g.t) + 4 + g.jy[i]];
+                g.ly[i] = A.lw_y[4 * ((long long)i * A.N + g.t) + g.jy[i]];
 #pragma unroll
                 for (int a = 0; a < N1; ++a) g.gy[i][a] = row[a];
             } else {
-                g.lx[i] = A.lw[8 * ((long long)(N1 * i) * A.N + g.t) + g.jx[i]];
+                g.lx[i] = A.lw_x[4 * ((long long)i * A.N + g.t) + g.jx[i]];
 #pragma unroll
                 for (int a = 0; a < N1; ++a) g.gx[i][a] = row[a];
             }
@@ -792,7 +803,8 @@ constexpr int ADJ_TY = 8;  // staged phase A tile: 32 x 8 targets (0.8 % faster 
 // gather's per-(population, target) stencil origin and weights, and 1 / s*.
 template <int N1>
 __global__ void __launch_bounds__(32 * ADJ_TY, 1)
-k_adjoint_jvp_staged(AdjArgs A, int wwa, int wha, double c_max, double* __restrict__ jvp) {
+k_adjoint_jvp_staged(AdjArgs A, int wwa, int wha, double c_max, double* __restrict__ jvp,
+                     const unsigned int* __restrict__ redo) {
     constexpr int TX = 32, NT = TX * ADJ_TY, Q = N1 * N1;
     extern __shared__ __align__(32) unsigned char smem_raw[];
     Double4* s_f = reinterpret_cast<Double4*>(smem_raw);  // [N1][WN]
@@ -801,8 +813,13 @@ k_adjoint_jvp_staged(AdjArgs A, int wwa, int wha, double c_max, double* __restri
     const int WN = wwa * wha;
     const int tid = threadIdx.x;
     const int tiles_x = (A.nx + TX - 1) / TX;
-    const int tx0 = (int)(blockIdx.x % tiles_x) * TX;
-    const int ty0 = (int)(blockIdx.x / tiles_x) * ADJ_TY;
+    // the tiles that k_adjoint_jvp_fixed left: {count, tiles}
+    const unsigned int left = redo[0];
+    for (unsigned int it = blockIdx.x; it < left; it += gridDim.x) {
+    __syncthreads();  // the last tile's staged rows are done with
+    const int tile = (int)redo[1 + it];
+    const int tx0 = tile % tiles_x * TX;
+    const int ty0 = tile / tiles_x * ADJ_TY;
     const int X = tx0 + tid % TX, Y = ty0 + tid / TX;
     const bool valid = X < A.nx && Y < A.ny;
     const long long node = (long long)Y * A.nx + X;
@@ -847,7 +864,7 @@ k_adjoint_jvp_staged(AdjArgs A, int wwa, int wha, double c_max, double* __restri
     stage_window<StagedAdj64, N1>(A.in, A.N, G, 0, wx0, wy0, ww, wh, WN, rux, ruy, rst, s_f,
                                   nullptr, tid, NT);
     __syncthreads();
-    if (!valid) return;
+    if (!valid) continue;
 
     const double inv = 1.0 / st;
     A.inv_st[node] = inv;
@@ -891,13 +908,18 @@ k_adjoint_jvp_staged(AdjArgs A, int wwa, int wha, double c_max, double* __restri
                 lagrange4_d(depy - fly + 1.0, ly[p], dly[p]);
                 top[p] = (int)fly - 1 - wy0;
                 in[p] = colok && top[p] >= 0 && top[p] + 3 < wh;
-                const long long o = (long long)(N1 * k + l) * A.N + node;
-                A.org[o] = make_int2((int)((long long)flx - 1 - X), (int)((long long)fly - 1 - Y));
-                double2* pw = reinterpret_cast<double2*>(A.lw + 8 * o);
-                pw[0] = make_double2(lx[0], lx[1]);
-                pw[1] = make_double2(lx[2], lx[3]);
-                pw[2] = make_double2(ly[p][0], ly[p][1]);
-                pw[3] = make_double2(ly[p][2], ly[p][3]);
+                if (l == 0) {
+                    A.org_x[(long long)k * A.N + node] = (int)((long long)flx - 1 - X);
+                    double2* pw = reinterpret_cast<double2*>(A.lw_x + 4 * ((long long)k * A.N + node));
+                    pw[0] = make_double2(lx[0], lx[1]);
+                    pw[1] = make_double2(lx[2], lx[3]);
+                }
+                if (k == 0) {
+                    A.org_y[(long long)l * A.N + node] = (int)((long long)fly - 1 - Y);
+                    double2* pw = reinterpret_cast<double2*>(A.lw_y + 4 * ((long long)l * A.N + node));
+                    pw[0] = make_double2(ly[p][0], ly[p][1]);
+                    pw[1] = make_double2(ly[p][2], ly[p][3]);
+                }
             }
             double Z[2][N1], Zux[2][N1], Zuy[2][N1], Zs[2][N1];
 #pragma unroll
@@ -1017,6 +1039,294 @@ k_adjoint_jvp_staged(AdjArgs A, int wwa, int wha, double c_max, double* __restri
             }
         }
     }
+    }
+}
+
+// Phase A with its contractions in fixed point (pond_fixed.cuh: the staged
+// window, its scale and range, the row sweep).  Each of the sums over a row's
+// sources that the three tangents need is one sweep of its own, with its
+// weights folded ahead of it,
+//   P = sum lx G_x g,  U = sum (-tau lx' G_x - lx G_x') g,
+//   S = sum (-c_k tau lx' G_x - lx G_x' xi) g    (tau = s dt; U, S times s),
+// so that the sweep's registers are the forward step's.  Per population, with
+// Z = sum_j ly P, D = sum_j ly' P,
+//   A = G_y Z,  dA/du_x = G_y sum ly U / s,  dA/du_y = -dt G_y D - G_y' Z / s,
+//   dA/ds = (G_y sum ly S - G_y' xi Z) / s - dt c_l G_y D.
+// Scales (units of R): P, Z 2^-60; U, G_y' Z, G_y' xi Z, D 2^-57; S 2^-56, with
+// tau <= 1.9 so that every sum stays below 2^63.  Tiles out of range go to
+// redo.  Also per target: the gather's stencil origins and weights (one set
+// per speed and direction) and 1 / s*.
+// Measured against k_adjoint_jvp_staged: see launch_adjoint_phase_a_staged.
+template <int N1, int TY>
+__global__ void __launch_bounds__(32 * TY, TY == 8 ? 1 : 2)
+k_adjoint_jvp_fixed(AdjArgs A, int wwa, int wha, double c_max_d, double* __restrict__ jvp,
+                    unsigned int* __restrict__ redo) {
+    constexpr int TX = 32, NT = TX * TY, Q = N1 * N1;
+    constexpr unsigned FULL = 0xffffffffu;
+    extern __shared__ __align__(32) unsigned char smem_raw[];
+    const int WN = wwa * wha;
+    int4* s_h = reinterpret_cast<int4*>(smem_raw);                // [N1][WN] high words
+    int4* s_l = s_h + (size_t)N1 * WN;                            // [N1][WN] low words
+    int2* s_gy = reinterpret_cast<int2*>(s_l + (size_t)N1 * WN);  // [Q][NT] y-map
+    int2* s_ly = s_gy + (size_t)Q * NT;                           // [4 N1][NT] y-weights
+    int2* s_dy = s_ly + (size_t)4 * N1 * NT;                      // [4 N1][NT] their derivatives, 2^57
+    __shared__ float s_red[4][NT / 32];
+    const Lattice& L = c_La[lattice_slot(N1)];
+    const LatticeFix& F = c_Lafix[lattice_slot(N1)];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int tiles_x = (A.nx + TX - 1) / TX;
+    const int tx0 = (int)(blockIdx.x % tiles_x) * TX;
+    const int ty0 = (int)(blockIdx.x / tiles_x) * TY;
+    const int X = tx0 + tid % TX, Y = ty0 + tid / TX;
+    const bool valid = X < A.nx && Y < A.ny;
+    const long long node = (long long)Y * A.nx + X;
+    const float c_max = (float)c_max_d;
+
+    // reference gauge and scale: the tile's centre node of the input state
+    const long long rnode = (long long)min(ty0 + TY / 2, A.ny - 1) * A.nx + min(tx0 + TX / 2, A.nx - 1);
+    const double rux = A.in.ux[rnode], ruy = A.in.uy[rnode], rst = A.in.st[rnode];
+    unsigned mh = 0u;
+    if (lane < Q) {
+        const int sh = fix_shift<N1>(lane / N1) + fix_shift<N1>(lane % N1);
+        mh = (unsigned)__double2hiint(fabs(A.in.f[(long long)lane * A.N + rnode]) * (double)(1 << sh));
+    }
+    mh = __reduce_max_sync(FULL, mh);
+    const int me = (int)(mh >> 20) - 1023, rexp = me + 5;
+    bool in_range = me > -900 && me < 900;
+
+    double ux = 0.0, uy = 0.0, st = 1.0;
+    float vxlo = 3.0e38f, vxhi = -3.0e38f, vylo = 3.0e38f, vyhi = -3.0e38f;
+    if (valid) {
+        ux = A.ux_s[node];
+        uy = A.uy_s[node];
+        st = A.st_s[node];
+        const float sp = (float)(c_max_d * st);
+        vxlo = (float)ux - sp;
+        vxhi = (float)ux + sp;
+        vylo = (float)uy - sp;
+        vyhi = (float)uy + sp;
+        const float de = fmaf(c_max, fabsf((float)(rst - st)),
+                              fmaxf(fabsf((float)(rux - ux)), fabsf((float)(ruy - uy))));
+        in_range = in_range && de <= kFixTileDe * (float)st && (float)(st * A.dt) <= 1.9f;
+    }
+    staged_block_minmax4<StagedAdj64, NT>(vxlo, vxhi, vylo, vyhi, s_red);
+    const float m = 1.0f, fdt = (float)A.dt;
+    const float bxl = fminf(fmaxf(vxlo, -1.0e6f), 1.0e6f), bxh = fminf(fmaxf(vxhi, -1.0e6f), 1.0e6f);
+    const float byl = fminf(fmaxf(vylo, -1.0e6f), 1.0e6f), byh = fminf(fmaxf(vyhi, -1.0e6f), 1.0e6f);
+    const int wx0 = (int)floorf((float)tx0 - bxh * fdt - m) - 1;
+    const int wx1 = (int)floorf((float)(tx0 + TX - 1) - bxl * fdt + m) + 2;
+    const int wy0 = (int)floorf((float)ty0 - byh * fdt - m) - 1;
+    const int wy1 = (int)floorf((float)(ty0 + TY - 1) - byl * fdt + m) + 2;
+    in_range = in_range && isfinite(vxlo) && isfinite(vxhi) && isfinite(vylo) && isfinite(vyhi) &&
+               fmaxf(fmaxf(fabsf(vxlo), fabsf(vxhi)), fmaxf(fabsf(vylo), fabsf(vyhi))) * fdt < 400.0f;
+    const int ww = max(1, min(wx1 - wx0 + 1, wwa)), wh = max(1, min(wy1 - wy0 + 1, wha));
+    GridDesc G;
+    G.nx = A.nx;
+    G.ny = A.ny;
+    G.offset = 0;
+    G.ix0 = 0;
+    G.iy0 = 0;
+    G.iw = A.nx;
+    G.ih = A.ny;
+    if (!__syncthreads_or(!in_range))
+        in_range = stage_window_fixed<N1, true>(A.in, A.N, G, 0, wx0, wy0, ww, wh, WN, rux, ruy, rst,
+                                                kFix - rexp, s_h, s_l, F, c_max, nullptr, tid, NT);
+    else
+        in_range = false;
+    if (__syncthreads_or(!in_range)) {  // also: the window is staged
+        // the FP64 kernel's tiles are 32 x ADJ_TY: a tile holds ADJ_TY / TY of these
+        if (tid == 0) {
+            const unsigned tile = (unsigned)(ty0 / ADJ_TY * tiles_x + tx0 / TX);
+            if (TY == ADJ_TY || atomicExch(redo + 1 + gridDim.x + tile, 1u) == 0u)
+                redo[1 + atomicAdd(redo, 1u)] = tile;
+        }
+        return;
+    }
+    if (!valid) return;
+
+    const double inv = 1.0 / st, inv60 = kFixOne / st, dt54 = A.dt * kFixDisplacement;
+    A.inv_st[node] = inv;
+    const long long rt = __double2ll_rn((rst - st) * inv60);
+    const long long dxt = __double2ll_rn((rux - ux) * inv60), dyt = __double2ll_rn((ruy - uy) * inv60);
+    const Fix Rt = fix_split(rt), tau = fix_split(__double2ll_rn(st * A.dt * (kFixOne / 8.0)));
+    Fix dex[N1], dey[N1];
+    int last[N1];  // the row that completes population l's stencil, else -1
+#pragma unroll
+    for (int a = 0; a < N1; ++a) {
+        const long long ca = fix_mul(F.c[a], Rt);
+        dex[a] = fix_split(dxt + ca);
+        dey[a] = fix_split(dyt + ca);
+    }
+    int lo = 0x7fffffff, hi = -1;
+#pragma unroll
+    for (int l = 0; l < N1; ++l) {
+        Fix ly[4], dy[4];
+        const int fy = fix_departure_d(__double2ll_rn(-fma(st, L.c[l], uy) * dt54), ly, dy);
+        const int top = Y - wy0 - 1 + fy;
+        last[l] = top >= 0 && top + 3 < wh ? top + 3 : -1;
+        if (last[l] >= 0) {
+            lo = min(lo, top);
+            hi = max(hi, top + 3);
+        }
+        A.org_y[(long long)l * A.N + node] = fy - 1;
+        double w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            s_ly[(4 * l + j) * NT + tid] = make_int2(ly[j].h, ly[j].l);
+            const Fix d8 = fix_split(((long long)dy[j].h * (1ll << 32) + dy[j].l) >> 3);
+            s_dy[(4 * l + j) * NT + tid] = make_int2(d8.h, d8.l);
+            w[j] = fix_to_double(ly[j]);
+        }
+        double2* pw = reinterpret_cast<double2*>(A.lw_y + 4 * ((long long)l * A.N + node));
+        pw[0] = make_double2(w[0], w[1]);
+        pw[1] = make_double2(w[2], w[3]);
+#pragma unroll
+        for (int b = 0; b < N1; ++b) {
+            const Fix gw = fix_gauge<N1>(F, l, b, dey[b]);
+            s_gy[(N1 * l + b) * NT + tid] = make_int2(gw.h, gw.l);
+        }
+    }
+    const double f_unit = pow2d(rexp - kFix);
+    constexpr double dn = 1.0 / (double)(1 << fix_shift<N1>(0));
+#pragma unroll 1
+    for (int k = 0; k < N1; ++k) {
+        Fix lx[4], dlx[4];
+        const int fx = fix_departure_d(__double2ll_rn(-fma(st, L.c[k], ux) * dt54), lx, dlx);
+        const int col = X - wx0 - 1 + fx;
+        A.org_x[(long long)k * A.N + node] = fx - 1;
+        double2* pw = reinterpret_cast<double2*>(A.lw_x + 4 * ((long long)k * A.N + node));
+        pw[0] = make_double2(fix_to_double(lx[0]), fix_to_double(lx[1]));
+        pw[1] = make_double2(fix_to_double(lx[2]), fix_to_double(lx[3]));
+        const bool on = col >= 0 && col + 3 < ww;
+        const double uk = k == 0 || k == N1 - 1 ? f_unit * dn : f_unit;
+        // mode 0: U, 1: S, 2: P (which completes what the others left)
+#pragma unroll 1
+        for (int mode = 0; on && mode < 3; ++mode) {
+            Fix cw[4][N1];
+#pragma unroll
+            for (int a = 0; a < N1; ++a) {
+                const Fix g = fix_gauge<N1>(F, k, a, dex[a]);
+                Fix gd{0, 0};
+                if (mode != 2) {
+                    long long d = fix_gauge_d<N1>(F, k, a, dex[a]);
+                    if (mode == 1) {
+                        const long long xi = ((long long)F.c[a].h * (1ll << 32) + F.c[a].l) +
+                                             ((long long)dex[a].h * (1ll << 32) + dex[a].l);
+                        d = fix_mul(fix_split(xi), fix_split(d));
+                    }
+                    gd = fix_split(d);
+                }
+#pragma unroll
+                for (int jx = 0; jx < 4; ++jx) {
+                    if (mode == 2) {
+                        cw[jx][a] = fix_split(fix_mul(lx[jx], g));
+                    } else {
+                        long long tb = fix_mul(fix_split(fix_mul(dlx[jx], g)), tau);
+                        long long lg = fix_mul(lx[jx], gd) >> 3;
+                        if (mode == 1) {
+                            tb = fix_mul(F.c[k], fix_split(tb)) >> 1;
+                            lg >>= 1;
+                        }
+                        cw[jx][a] = fix_split(-tb - lg);
+                    }
+                }
+            }
+            Fix Pb[4][N1];
+#pragma unroll 1
+            for (int y = lo; y <= hi; ++y) {
+                const int4* sh = s_h + y * ww + col;
+                const int4* sl = s_l + y * ww + col;
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+#pragma unroll
+                    for (int b = 0; b < N1; ++b) Pb[i][b] = Pb[i + 1][b];
+                long long h[4], mm[4];
+#pragma unroll
+                for (int b = 0; b < 4; ++b) h[b] = mm[b] = 0;
+#pragma unroll
+                for (int jx = 0; jx < 4; ++jx) {
+#pragma unroll
+                    for (int a = 0; a < N1; ++a) {
+                        const int4 gh = sh[(size_t)a * WN + jx], gl = sl[(size_t)a * WN + jx];
+                        fix_mad(cw[jx][a], gh.x, gl.x, h[0], mm[0]);
+                        fix_mad(cw[jx][a], gh.y, gl.y, h[1], mm[1]);
+                        fix_mad(cw[jx][a], gh.z, gl.z, h[2], mm[2]);
+                        if (N1 == 4) fix_mad(cw[jx][a], gh.w, gl.w, h[3], mm[3]);
+                    }
+                }
+#pragma unroll
+                for (int b = 0; b < N1; ++b) Pb[3][b] = fix_split(fix_sum(h[b], mm[b]));
+                unsigned todo = 0u;
+#pragma unroll
+                for (int l = 0; l < N1; ++l) todo |= y == last[l] ? 1u << l : 0u;
+                while (todo) {
+                    const int l = __ffs(todo) - 1;
+                    todo &= todo - 1;
+                    long long fh = 0, fm = 0, eh = 0, em = 0, ph = 0, pm = 0, qh = 0, qm = 0;
+                    Fix ly[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int2 v = s_ly[(4 * l + j) * NT + tid];
+                        ly[j] = Fix{v.x, v.y};
+                    }
+#pragma unroll
+                    for (int b = 0; b < N1; ++b) {
+                        long long zh = 0, zm = 0;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) fix_mad(ly[j], Pb[j][b].h, Pb[j][b].l, zh, zm);
+                        const Fix z = fix_split(fix_sum(zh, zm));
+                        const int2 v = s_gy[(N1 * l + b) * NT + tid];
+                        const Fix gw{v.x, v.y};
+                        fix_mad(gw, z.h, z.l, fh, fm);  // G_y sum ly (P, U or S)
+                        if (mode == 2) {
+                            long long dh = 0, dm = 0;
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const int2 w = s_dy[(4 * l + j) * NT + tid];
+                                fix_mad(Fix{w.x, w.y}, Pb[j][b].h, Pb[j][b].l, dh, dm);
+                            }
+                            const Fix d = fix_split(fix_sum(dh, dm));
+                            fix_mad(gw, d.h, d.l, eh, em);  // G_y D
+                            const long long gd = fix_gauge_d<N1>(F, l, b, dey[b]);
+                            const long long xi = ((long long)F.c[b].h * (1ll << 32) + F.c[b].l) +
+                                                 ((long long)dey[b].h * (1ll << 32) + dey[b].l);
+                            const long long gx = fix_mul(fix_split(xi), fix_split(gd));
+                            fix_mad(fix_split(gd >> 3), z.h, z.l, ph, pm);  // G_y' Z
+                            fix_mad(fix_split(gx >> 3), z.h, z.l, qh, qm);  // G_y' xi Z
+                        }
+                    }
+                    const long long q = (long long)(N1 * k + l) * A.N + node;
+                    const long long plane = (long long)Q * A.N;
+                    const double u = l == 0 || l == N1 - 1 ? uk * dn : uk;
+                    const double f = (double)fix_sum(fh, fm);
+                    if (mode == 0) {
+                        jvp[plane + q] = f * (8.0 * u * inv);
+                    } else if (mode == 1) {
+                        jvp[3 * plane + q] = f * (16.0 * u * inv);
+                    } else {
+                        jvp[q] = f * u;
+                        const double d = (double)fix_sum(eh, em) * (8.0 * u * A.dt);
+                        const double ui = 8.0 * u * inv;
+                        jvp[2 * plane + q] = -fma((double)fix_sum(ph, pm), ui, d);
+                        const double qx = fma((double)fix_sum(qh, qm), ui, L.c[l] * d);
+                        jvp[3 * plane + q] -= qx;
+                    }
+                }
+            }
+        }
+        // stencils off the window
+#pragma unroll 1
+        for (int l = 0; l < N1; ++l) {
+            int la = last[0];
+#pragma unroll
+            for (int i = 1; i < N1; ++i) la = i == l ? last[i] : la;
+            if (on && la >= 0) continue;
+            double R[4];
+            adj_population_direct<N1>(A, X, Y, k, l, ux, uy, st, R);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) jvp[((long long)i * Q + N1 * k + l) * A.N + node] = R[i];
+        }
+    }
 }
 
 // The rest of phase A from A* and its tangents: the collision cotangent,
@@ -1109,26 +1419,60 @@ __global__ void __launch_bounds__(256) k_adjoint_epilogue(AdjArgs A, const doubl
     if ((threadIdx.x & 31) == 0) atomicAdd(A.beta_bar, bb);
 }
 
-// Shared memory and launch of the staged phase A for a window of wwa x wha
-// staged nodes (FP64 rows of 32 bytes).
-cudaError_t launch_adjoint_phase_a_staged(const AdjArgs& A, int n1, int wwa, int wha, double c_max,
-                                          double* jvp, cudaStream_t s) {
-    static int s_set[64][2] = {{0}};
+// Launch of the staged phase A: the fixed-point kernel, the FP64 kernel over the
+// tiles it left (windows of wwa x wha staged nodes), the epilogue.  The fixed
+// kernel takes 32 x 8 tiles, or 32 x 4 where the window of those does not fit.
+// 256^2: 2.12 ms for the FP64 kernel alone, 0.44 ms so (4 steps forward and back:
+// 21.6 -> 14.9 ms).
+cudaError_t launch_adjoint_phase_a_staged(const AdjArgs& A, int n1, int ex, int ey, double c_max,
+                                          double* jvp, unsigned int* redo, int sms, cudaStream_t s) {
+    static int s_set[64][2] = {{0}}, s_fix[64][4] = {{0}};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    const size_t smem = (size_t)n1 * wwa * wha * sizeof(Double4);
-    void (*kern)(AdjArgs, int, int, double, double*) =
-        n1 == 3 ? k_adjoint_jvp_staged<3> : k_adjoint_jvp_staged<4>;
-    int& set = s_set[dev][n1 == 3 ? 1 : 0];
-    if ((int)smem > set) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        set = (int)smem;
+    auto raise = [](const void* kern, size_t smem, int* set) {
+        if ((int)smem <= *set) return cudaSuccess;
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess) *set = (int)smem;
+        return e;
+    };
+    const size_t cap = 220 * 1024, cap64 = 200 * 1024;
+    int ty = 8, w = 32 + ex, h = 8 + ey;
+    auto bytes = [&] { return (size_t)n1 * w * h * 32 + (size_t)32 * ty * 8 * (n1 * n1 + 8 * n1); };
+    if (bytes() > cap) {
+        ty = 4;
+        h = 4 + ey;
     }
-    const unsigned tiles = (unsigned)(((A.nx + 31) / 32) * ((A.ny + ADJ_TY - 1) / ADJ_TY));
-    kern<<<tiles, 32 * ADJ_TY, smem, s>>>(A, wwa, wha, c_max, jvp);
+    while (bytes() > cap) {
+        if (w - 32 >= h - ty) --w; else --h;
+    }
+    const long long tiles_x = (A.nx + 31) / 32, tiles = tiles_x * ((A.ny + ty - 1) / ty);
+    const long long tiles8 = tiles_x * ((A.ny + ADJ_TY - 1) / ADJ_TY);
+    void (*fixed)(AdjArgs, int, int, double, double*, unsigned int*) =
+        n1 == 3 ? (ty == 8 ? k_adjoint_jvp_fixed<3, 8> : k_adjoint_jvp_fixed<3, 4>)
+                : (ty == 8 ? k_adjoint_jvp_fixed<4, 8> : k_adjoint_jvp_fixed<4, 4>);
+    e = raise((const void*)fixed, bytes(), &s_fix[dev][(n1 == 3 ? 2 : 0) + (ty == 8 ? 1 : 0)]);
+    // the count, and (32 x 4) the marks behind the list
+    if (e == cudaSuccess) e = cudaMemsetAsync(redo, 0, sizeof(unsigned int), s);
+    if (e == cudaSuccess && ty != ADJ_TY)
+        e = cudaMemsetAsync(redo + 1 + tiles, 0, sizeof(unsigned int) * tiles8, s);
+    if (e != cudaSuccess) return e;
+    fixed<<<(unsigned)tiles, 32 * ty, bytes(), s>>>(A, w, h, c_max, jvp, redo);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+
+    w = 32 + ex;
+    h = ADJ_TY + ey;
+    while ((size_t)n1 * w * h * sizeof(Double4) > cap64) {
+        if (w - 32 >= h - ADJ_TY) --w; else --h;
+    }
+    const size_t smem = (size_t)n1 * w * h * sizeof(Double4);
+    void (*kern)(AdjArgs, int, int, double, double*, const unsigned int*) =
+        n1 == 3 ? k_adjoint_jvp_staged<3> : k_adjoint_jvp_staged<4>;
+    e = raise((const void*)kern, smem, &s_set[dev][n1 == 3 ? 1 : 0]);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)(tiles8 < sms ? tiles8 : sms), 32 * ADJ_TY, smem, s>>>(A, w, h, c_max, jvp, redo);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const unsigned nb = (unsigned)((A.N + 255) / 256);
@@ -1166,6 +1510,9 @@ void destroy_adjoint(pond_ctx* ctx) {
     cudaFree(a->minmax);
     cudaFree(a->org);
     cudaFree(a->lw);
+    cudaFree(a->org1);
+    cudaFree(a->lw1);
+    cudaFree(a->redo);
     cudaFree(a->inv_st);
     cudaFree(a->jvp);
     cudaFree(a->nu_dev);
@@ -1277,10 +1624,19 @@ static pond_status adjoint_step_impl(pond_ctx* ctx, const double* const out_gaug
         ACK(cudaMalloc(&a->nu_dev, sizeof(double)), "adjoint alloc");
         ACK(cudaMemsetAsync(a->nu_dev, 0, sizeof(double), ctx->stream), "adjoint alloc");
         ACK(cudaMalloc(&a->minmax, sizeof(double) * 6), "adjoint alloc");
-        ACK(cudaMalloc(&a->org, sizeof(int2) * 16 * N), "adjoint alloc");
-        ACK(cudaMalloc(&a->lw, sizeof(double) * 8 * 16 * N), "adjoint alloc");
-        ACK(cudaMalloc(&a->inv_st, sizeof(double) * N), "adjoint alloc");
         if (fp64) {
+            ACK(cudaMalloc(&a->inv_st, sizeof(double) * N), "adjoint alloc");
+            if (ctx_staged(ctx)) {
+                // the list and marks of the finer (32 x 4) tiles
+                const GridDesc& G0 = ctx->grids_host[0];
+                const size_t tiles = ((size_t)(G0.nx + 31) / 32) * (((size_t)G0.ny + 3) / 4);
+                ACK(cudaMalloc(&a->org1, sizeof(int) * 2 * 4 * N), "adjoint alloc");
+                ACK(cudaMalloc(&a->lw1, sizeof(double) * 2 * 4 * 4 * N), "adjoint alloc");
+                ACK(cudaMalloc(&a->redo, sizeof(unsigned int) * (1 + 2 * tiles)), "adjoint alloc");
+            } else {
+                ACK(cudaMalloc(&a->org, sizeof(int2) * 16 * N), "adjoint alloc");
+                ACK(cudaMalloc(&a->lw, sizeof(double) * 8 * 16 * N), "adjoint alloc");
+            }
             ACK(cudaMalloc(&a->fwd.f, sizeof(double) * 16 * N), "adjoint alloc");
             ACK(cudaMalloc(&a->fwd.ux, sizeof(double) * N), "adjoint alloc");
             ACK(cudaMalloc(&a->fwd.uy, sizeof(double) * N), "adjoint alloc");
@@ -1339,6 +1695,10 @@ static pond_status adjoint_step_impl(pond_ctx* ctx, const double* const out_gaug
     A.beta_bar = a->beta_bar;
     A.org = a->org;
     A.lw = a->lw;
+    A.org_x = a->org1;
+    A.org_y = a->org1 ? a->org1 + 4 * N : nullptr;
+    A.lw_x = a->lw1;
+    A.lw_y = a->lw1 ? a->lw1 + 16 * N : nullptr;
     A.inv_st = a->inv_st;
     A.nx = G.nx;
     A.ny = G.ny;
@@ -1359,19 +1719,15 @@ static pond_status adjoint_step_impl(pond_ctx* ctx, const double* const out_gaug
     const unsigned nb = (unsigned)((N + ADJ_WARPS - 1) / ADJ_WARPS);
     nvtxRangePushA("adjoint targets + transpose gather");
     if (ctx_staged(ctx)) {
-        // phase A in the staged form: a window per 32 x 4 tile of targets
-        // sized from the bounds of the particle velocities at lambda*
+        // phase A in the staged form: a window per tile of targets sized from the bounds of the particle velocities at lambda*
         if (!a->jvp) ACK(cudaMalloc(&a->jvp, sizeof(double) * 4 * 16 * N), "adjoint alloc");
         const double cm = ctx->L.c_max;
         const double sx = (mm[1] - mm[0]) + 2.0 * cm * mm[5];
         const double sy = (mm[3] - mm[2]) + 2.0 * cm * mm[5];
-        int wwa = 32 + window_extent(sx, A.dt, 2.0) + 5;
-        int wha = ADJ_TY + window_extent(sy, A.dt, 2.0) + 5;
-        const size_t cap = 200 * 1024;
-        while ((size_t)ctx->L.n1 * wwa * wha * sizeof(Double4) > cap) {
-            if (wwa - 32 >= wha - ADJ_TY) --wwa; else --wha;
-        }
-        ACK(launch_adjoint_phase_a_staged(A, ctx->L.n1, wwa, wha, cm, a->jvp, s),
+        int sms = 0;
+        ACK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device), "SM count");
+        ACK(launch_adjoint_phase_a_staged(A, ctx->L.n1, window_extent(sx, A.dt, 2.0) + 5,
+                                          window_extent(sy, A.dt, 2.0) + 5, cm, a->jvp, a->redo, sms, s),
             "adjoint targets (staged)");
     } else {
         if (ctx->L.n1 == 3) k_adjoint_targets<3><<<nb, ADJ_WARPS * 32, 0, s>>>(A);

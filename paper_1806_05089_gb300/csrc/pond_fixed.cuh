@@ -156,6 +156,38 @@ __device__ __forceinline__ int fix_departure(long long d, Fix (&l)[4]) {
     return (int)(d >> 54);
 }
 
+// fix_departure with the derivatives of the cubic weights by t, dl.
+__device__ __forceinline__ int fix_departure_d(long long d, Fix (&l)[4], Fix (&dl)[4]) {
+    const long long s = (d & ((1ll << 54) - 1)) << (kFix - 54), one = 1ll << kFix;
+    const Fix S = fix_split(s), sixth = fix_split((one + 3) / 6);
+    const Fix V = fix_split(fix_mul(sixth, fix_split(fix_mul(S, fix_split(one - s)))));
+    const long long v = (long long)V.h * (1ll << 32) + V.l, w = fix_mul(S, V);
+    l[0] = fix_split(w - 2 * v);
+    l[1] = fix_split(one - s + 3 * (v - w));
+    l[2] = fix_split(s + 3 * w);
+    l[3] = fix_split(-(v + w));
+    // v' = (1 - 2 s) / 6, w' = v' s + v
+    const long long dv = fix_mul(sixth, fix_split(one - 2 * s)), dw = fix_mul(S, fix_split(dv)) + v;
+    dl[0] = fix_split(dw - 2 * dv);
+    dl[1] = fix_split(3 * (dv - dw) - one);
+    dl[2] = fix_split(one + 3 * dw);
+    dl[3] = fix_split(-(dv + dw));
+    return (int)(d >> 54);
+}
+
+// The derivative of fix_gauge's entry by its offset.
+template <int N1>
+__device__ __forceinline__ long long fix_gauge_d(const LatticeFix& F, int k, int a, Fix de) {
+    long long t = 2 * F.d2[k][a];
+    if (N1 == 4) t += 3 * fix_mul(F.d3[k][a], de);
+    return F.d1[k][a] + fix_mul(de, fix_split(t));
+}
+
+// A weight as a double.
+__device__ __forceinline__ double fix_to_double(Fix w) {
+    return (double)((long long)w.h * (1ll << 32) + w.l) * (1.0 / kFixOne);
+}
+
 // 2^e for |e| < 1000.
 __device__ __forceinline__ double pow2d(int e) {
     return __hiloint2double((1023 + e) << 20, 0);

@@ -127,3 +127,29 @@ def test_allocation_free_step_matches_the_context_step(name, nx, ny, lattice):
     assert stats["nonphysical"] == 0 and stats["halo_fallback"] == 0
     for a, b in zip(out, (want.f, want.ux, want.uy, want.T)):
         assert np.array_equal(a.cpu().numpy(), b)
+
+
+@pytest.mark.parametrize("lattice", [pond.POND_D2Q16, pond.POND_D2Q9])
+@pytest.mark.parametrize("name,nx,ny,hot", [("plain", 33, 9, 1.0), ("plain", 70, 30, 3.0),
+                                            ("plain", 70, 30, 6.0), ("density", 160, 12, 1.0),
+                                            ("shear", 40, 64, 1.0)])
+def test_adjoint_step_matches_the_direct_kernels(name, nx, ny, hot, lattice):
+    """Tiles in and out of the fixed-point tangents' range (gauge spread,
+    magnitudes, tau > 1.9 at T = 6), the 32 x 4 tiles of wide windows, against
+    the per-pair kernels; 1e-9 of the largest, as the adjoint's other checks."""
+    import torch
+    T_L = 1.0 / 3.0 if lattice == pond.POND_D2Q9 else 1.0
+    fields = field(name, nx, ny, T_L)
+    Q = 9 if lattice == pond.POND_D2Q9 else 16
+    rng = np.random.default_rng(5)
+    fbar = torch.tensor(rng.standard_normal((Q, ny, nx)), device="cuda")
+    gbar = torch.tensor(rng.standard_normal((3, ny, nx)), device="cuda")
+    got = []
+    for kernel in (pond.POND_KERNEL_STAGED, pond.POND_KERNEL_DIRECT):
+        with pond.Sim(nx, ny, pond.POND_FP64, lattice=lattice, T_ref=T_L, kernel=kernel) as s:
+            s.set_state(fields.rho, fields.ux, fields.uy, hot * fields.T)
+            out = torch.empty_like(fbar), torch.empty_like(gbar)
+            nu = pond.pond_adjoint_step(s.ctx, fbar, gbar, *out)
+            got.append([a.cpu().numpy() for a in out] + [np.array(nu)])
+    for a, b in zip(*got):
+        assert np.abs(a - b).max() <= 1e-9 * np.abs(b).max()
