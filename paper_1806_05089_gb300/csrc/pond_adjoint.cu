@@ -41,16 +41,19 @@ namespace pond {
 
 // Lattice constants of the adjoint kernels, slot lattice_slot(n1).
 __constant__ Lattice c_La[2];
-__constant__ LatticeFix c_Lafix[2];
+__constant__ LatticeFix c_Lafix[2], c_Lafix1[2];  // scaled, and not
 
 cudaError_t upload_lattice_adjoint() {
     const Lattice L[2] = {make_lattice(POND_D2Q16), make_lattice(POND_D2Q9)};
     const LatticeFix F[2] = {make_lattice_fix(L[0]), make_lattice_fix(L[1])};
     cudaError_t e = cudaMemcpyToSymbol(c_La, L, sizeof(L));
+    const LatticeFix F1[2] = {make_lattice_fix(L[0], false), make_lattice_fix(L[1], false)};
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_Lafix, F, sizeof(F));
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_Lafix1, F1, sizeof(F1));
     return e;
 }
 
+struct ScatterTile;
 struct AdjointScratch {
     int64_t N = 0;
     StateBuf<double> fwd{};   // forward step output: gauge = lambda*
@@ -64,7 +67,9 @@ struct AdjointScratch {
     // staged contexts keep org and lw per speed and direction instead
     int* org1 = nullptr;         // [2][4][N]
     double* lw1 = nullptr;       // [2][4][N][4]
-    unsigned int* redo = nullptr;  // phase A: {count, tiles, marks} left to the FP64 kernel
+    unsigned int* redo = nullptr;  // {count, tiles, marks} left to the FP64 kernels (phase A, then B)
+    double* win = nullptr;         // phase B: the tiles' windows of f_bar
+    ScatterTile* tiles = nullptr;
     double* inv_st = nullptr;    // [N] 1 / s* at every target
     double* jvp = nullptr;       // [4][16][N] A*, dA/du_x, dA/du_y, dA/ds (staged phase A)
     double* nu_dev = nullptr;    // nu cotangent of calls with nu_bar_accum == NULL
@@ -118,6 +123,7 @@ struct AdjArgs {
 };
 
 constexpr int ADJ_WARPS = 4;
+constexpr int ADJ_TY = 8;  // tiles of targets of the staged kernels: 32 x 8
 
 template <int N1>
 __global__ void __launch_bounds__(ADJ_WARPS * 32, 2) k_adjoint_targets(AdjArgs A) {
@@ -433,19 +439,24 @@ struct GatherSlot {
 };
 
 template <int N1>
-__global__ void __launch_bounds__(ADJ_GATHER_WARPS * 32) k_adjoint_sources_t(AdjArgs A) {
+__global__ void __launch_bounds__(ADJ_GATHER_WARPS * 32)
+k_adjoint_sources_t(AdjArgs A, const unsigned int* __restrict__ left) {
     constexpr int Q = N1 * N1;
     constexpr unsigned FULL = 0xffffffffu;
+    // only the targets of the tiles that k_adjoint_scatter left (left: {count,
+    // a mark per tile}), added to what its reduction stored
+    if (left[0] == 0u) return;
+    const int tiles_x = (A.nx + 31) / 32;
     __shared__ GatherSlot s_slot[ADJ_GATHER_WARPS][32];
     __shared__ unsigned short s_hit[ADJ_GATHER_WARPS][32 * Q];
     __shared__ unsigned short s_job[ADJ_GATHER_WARPS][32 * 2 * N1];
     const Lattice& L = c_La[lattice_slot(N1)];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const long long src = (long long)blockIdx.x * ADJ_GATHER_WARPS + wid;
-    if (src >= A.N) return;  // warp-uniform
+    GatherSlot& my = s_slot[wid][lane];
+    for (long long src = (long long)blockIdx.x * ADJ_GATHER_WARPS + wid; src < A.N;
+         src += (long long)gridDim.x * ADJ_GATHER_WARPS) {  // warp-uniform
     const int JX = (int)(src % A.nx), JY = (int)(src / A.nx);
     const double uxj = A.in.ux[src], uyj = A.in.uy[src], stj = A.in.st[src];
-    GatherSlot& my = s_slot[wid][lane];
     unsigned short* hitq = s_hit[wid];
     unsigned short* jobq = s_job[wid];
 
@@ -472,9 +483,10 @@ __global__ void __launch_bounds__(ADJ_GATHER_WARPS * 32) k_adjoint_sources_t(Adj
         // 1. this lane's candidate: its hit set K x L and gauge offsets
         const int c = c0 + lane;
         unsigned kmask = 0u, lmask = 0u;
-        if (c < nc) {
-            const int xx = JX + xlo + c % wx, yy = JY + ylo + c / wx;
-            const long long t = (long long)wrap_idx(yy, A.ny) * A.nx + wrap_idx(xx, A.nx);
+        const int xx = JX + xlo + c % wx, yy = JY + ylo + c / wx;
+        const int wy_ = wrap_near(yy, A.ny), wx_ = wrap_near(xx, A.nx);
+        if (c < nc && left[1 + wy_ / ADJ_TY * tiles_x + wx_ / 32] != 0u) {
+            const long long t = (long long)wy_ * A.nx + wx_;
 #pragma unroll
             for (int i = 0; i < N1; ++i) {
                 const int jx = JX - (xx + A.org_x[(long long)i * A.N + t]);
@@ -588,7 +600,7 @@ __global__ void __launch_bounds__(ADJ_GATHER_WARPS * 32) k_adjoint_sources_t(Adj
         pux = tot * gxu;
         puy = tot * gyu;
         pst = tot * (gsx + gsy);
-        A.fbar_in[(long long)p * A.N + src] = tot;
+        A.fbar_in[(long long)p * A.N + src] += tot;
     }
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -598,10 +610,11 @@ __global__ void __launch_bounds__(ADJ_GATHER_WARPS * 32) k_adjoint_sources_t(Adj
     }
     if (lane == 0) {
         const double is = 1.0 / stj;
-        A.gbar_in[src] = pux * is;
-        A.gbar_in[A.N + src] = puy * is;
+        A.gbar_in[src] += pux * is;
+        A.gbar_in[A.N + src] += puy * is;
         // s = sqrt(T / T_L): dL/dT = dL/ds / (2 s T_L)
-        A.gbar_in[2 * A.N + src] = pst * is / (2.0 * stj * A.T_L);
+        A.gbar_in[2 * A.N + src] += pst * is / (2.0 * stj * A.T_L);
+    }
     }
 }
 
@@ -797,7 +810,6 @@ __device__ __noinline__ void adj_population_direct(const AdjArgs& A, int X, int 
     out4[3] = dAst;
 }
 
-constexpr int ADJ_TY = 8;  // staged phase A tile: 32 x 8 targets (0.8 % faster than 32 x 4)
 
 // Phase A, staged: A*, its tangents at lambda* into jvp[4][Q][N], the
 // gather's per-(population, target) stencil origin and weights, and 1 / s*.
@@ -1481,6 +1493,382 @@ cudaError_t launch_adjoint_phase_a_staged(const AdjArgs& A, int n1, int ex, int 
     return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------------------
+// Phase B in fixed point.  Per source and target the gather evaluates gauge maps
+// and visits some 80 targets; the transpose of the staged reconstruction
+// instead runs over the targets, in the frame of their tile's reference gauge r:
+//   h(s)[a][b] = sum_{t, k} lx_k(s) G_x(r -> t)[k][a] V_k(y_s)[b],
+//   V_k(y)[b]  = sum_l ly_l(y) w_(k,l) G_y(r -> t)[l][b]  over the stencils with row y,
+// 2304 products per target (D2Q16) as in a pass of the step, scattered into
+// the tile's window of sources in shared memory.  The sums are 64-bit integers
+// (the largest |w| of the tile is held to 2^55 .. 2^56; every sum of a source
+// stays below 2^63), added as two 32-bit atomics with the carry taken from the
+// first one's result, so their order does not matter and the result is the
+// same in every run.  (A 64-bit shared-memory atomic takes 14.6 clocks per warp
+// and SM, two 32-bit ones 3 to 4.)  Then each source's h is taken back to its
+// own frame, G(s -> r)^T h, in FP64, and stored per tile; k_adjoint_reduce adds the
+// tiles that reach a source in a fixed order and forms the gauge cotangent.
+// Tiles whose gauges, displacements or cotangents are out of range, or with a
+// stencil off the window, are marked and left to k_adjoint_sources_t.
+struct ScatterTile {
+    int x0, y0, w, h;  // the window in unwrapped coordinates; w = 0: left
+};
+constexpr int ADJ_SCATTER_WN = 1248;  // window nodes (160 KB of sums on D2Q16)
+
+__device__ __forceinline__ void atomic_add64(unsigned int* lo, unsigned int* hi, long long v) {
+    const unsigned int vl = (unsigned int)v;
+    const unsigned int old = atomicAdd(lo, vl);
+    atomicAdd(hi, (unsigned int)((unsigned long long)v >> 32) + (old + vl < old ? 1u : 0u));
+}
+
+template <int N1>
+__global__ void __launch_bounds__(32 * ADJ_TY, 1)
+k_adjoint_scatter(AdjArgs A, double c_max_d, double* __restrict__ win, ScatterTile* __restrict__ tiles,
+                  unsigned int* __restrict__ left) {
+    constexpr int TX = 32, TY = ADJ_TY, NT = TX * TY, Q = N1 * N1, WN = ADJ_SCATTER_WN;
+    constexpr unsigned FULL = 0xffffffffu;
+    extern __shared__ __align__(32) unsigned char smem_raw[];
+    unsigned int* s_lo = reinterpret_cast<unsigned int*>(smem_raw);  // [Q][WN]
+    unsigned int* s_hi = s_lo + (size_t)Q * WN;                      // [Q][WN]
+    int2* s_gy = reinterpret_cast<int2*>(s_hi + (size_t)Q * WN);     // [Q][NT] G_y(r -> t)
+    int2* s_ly = s_gy + (size_t)Q * NT;                              // [4 N1][NT] y-weights
+    __shared__ float s_red[4][NT / 32];
+    __shared__ unsigned int s_max;
+    const Lattice& L = c_La[lattice_slot(N1)];
+    const LatticeFix& F = c_Lafix1[lattice_slot(N1)];
+    const int tid = threadIdx.x;
+    const int tiles_x = (A.nx + TX - 1) / TX;
+    const int tx0 = (int)(blockIdx.x % tiles_x) * TX, ty0 = (int)(blockIdx.x / tiles_x) * TY;
+    const int X = tx0 + tid % TX, Y = ty0 + tid / TX;
+    const bool valid = X < A.nx && Y < A.ny;
+    const long long node = (long long)Y * A.nx + X, N = A.N;
+    const float c_max = (float)c_max_d;
+    if (tid == 0) s_max = 0u;
+    const long long rnode = (long long)min(ty0 + TY / 2, A.ny - 1) * A.nx + min(tx0 + TX / 2, A.nx - 1);
+    const double rux = A.in.ux[rnode], ruy = A.in.uy[rnode], rst = A.in.st[rnode];
+
+    bool in_range = true;
+    double ux = 0.0, uy = 0.0, st = 1.0;
+    unsigned int mh = 0u;
+    float vxlo = 3.0e38f, vxhi = -3.0e38f, vylo = 3.0e38f, vyhi = -3.0e38f;
+    if (valid) {
+        ux = A.ux_s[node];
+        uy = A.uy_s[node];
+        st = A.st_s[node];
+        const float sp = (float)(c_max_d * st);
+        vxlo = (float)ux - sp;
+        vxhi = (float)ux + sp;
+        vylo = (float)uy - sp;
+        vyhi = (float)uy + sp;
+        const float de = fmaf(c_max, fabsf((float)(rst - st)),
+                              fmaxf(fabsf((float)(rux - ux)), fabsf((float)(ruy - uy))));
+        in_range = de <= kFixTileDe * (float)st;
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+            mh = max(mh, (unsigned)__double2hiint(A.w[(long long)q * N + node]) & 0x7fffffffu);
+    }
+    mh = __reduce_max_sync(FULL, mh);
+    staged_block_minmax4<StagedAdj64, NT>(vxlo, vxhi, vylo, vyhi, s_red);  // (orders s_max = 0)
+    if ((tid & 31) == 0) atomicMax(&s_max, mh);
+    const float m = 1.0f, fdt = (float)A.dt;
+    const float bxl = fminf(fmaxf(vxlo, -1.0e6f), 1.0e6f), bxh = fminf(fmaxf(vxhi, -1.0e6f), 1.0e6f);
+    const float byl = fminf(fmaxf(vylo, -1.0e6f), 1.0e6f), byh = fminf(fmaxf(vyhi, -1.0e6f), 1.0e6f);
+    const int wx0 = (int)floorf((float)tx0 - bxh * fdt - m) - 1;
+    const int wx1 = (int)floorf((float)(tx0 + TX - 1) - bxl * fdt + m) + 2;
+    const int wy0 = (int)floorf((float)ty0 - byh * fdt - m) - 1;
+    const int wy1 = (int)floorf((float)(ty0 + TY - 1) - byl * fdt + m) + 2;
+    const int ww = max(1, min(wx1 - wx0 + 1, WN)), wh = max(1, min(wy1 - wy0 + 1, WN / ww));
+    in_range = in_range && isfinite(vxlo) && isfinite(vxhi) && isfinite(vylo) && isfinite(vyhi) &&
+               fmaxf(fmaxf(fabsf(vxlo), fabsf(vxhi)), fmaxf(fabsf(vylo), fabsf(vyhi))) * fdt < 400.0f;
+    __syncthreads();
+    mh = s_max;
+    // the scale: |w| 2^scale < 2^56 (all zero: any)
+    const int scale = mh == 0u ? 0 : 55 - ((int)(mh >> 20) - 1023);
+    in_range = in_range && mh < 0x7ff00000u && (mh == 0u || (scale > -900 && scale < 900));
+
+    // this target's map and stencils (all in the window, or the tile is left)
+    const double inv60 = kFixOne / st, dt54 = A.dt * kFixDisplacement;
+    const long long rt = __double2ll_rn((rst - st) * inv60);
+    const long long dxt = __double2ll_rn((rux - ux) * inv60), dyt = __double2ll_rn((ruy - uy) * inv60);
+    const Fix Rt = fix_split(rt);
+    Fix dex[N1];
+    int top[N1];
+    if (valid) {
+        Fix dey[N1];
+#pragma unroll
+        for (int a = 0; a < N1; ++a) {
+            const long long ca = fix_mul(F.c[a], Rt);
+            dex[a] = fix_split(dxt + ca);
+            dey[a] = fix_split(dyt + ca);
+        }
+#pragma unroll
+        for (int l = 0; l < N1; ++l) {
+            Fix w[4];
+            top[l] = Y - wy0 - 1 + fix_departure(__double2ll_rn(-fma(st, L.c[l], uy) * dt54), w);
+            const int col = X - wx0 - 1 + fix_departure(__double2ll_rn(-fma(st, L.c[l], ux) * dt54), w);
+            in_range = in_range && top[l] >= 0 && top[l] + 3 < wh && col >= 0 && col + 3 < ww;
+        }
+#pragma unroll
+        for (int l = 0; l < N1; ++l) {
+            Fix w[4];
+            fix_departure(__double2ll_rn(-fma(st, L.c[l], uy) * dt54), w);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s_ly[(4 * l + j) * NT + tid] = make_int2(w[j].h, w[j].l);
+#pragma unroll
+            for (int b = 0; b < N1; ++b) {
+                const Fix g = fix_gauge<N1>(F, l, b, dey[b]);
+                s_gy[(N1 * l + b) * NT + tid] = make_int2(g.h, g.l);
+            }
+        }
+    }
+    const int wn = ww * wh;
+    for (int i = tid; i < Q * WN; i += NT) s_lo[i] = s_hi[i] = 0u;
+    if (__syncthreads_or(!in_range)) {  // also: the sums are zero
+        if (tid == 0) {
+            tiles[blockIdx.x] = ScatterTile{0, 0, 0, 0};
+            left[1 + blockIdx.x] = 1u;
+            atomicAdd(left, 1u);
+        }
+        return;
+    }
+    if (tid == 0) {
+        tiles[blockIdx.x] = ScatterTile{wx0, wy0, ww, wh};
+        left[1 + blockIdx.x] = 0u;
+    }
+
+    if (valid) {
+        int lo = top[0], hi = top[0] + 3;
+#pragma unroll
+        for (int l = 1; l < N1; ++l) {
+            lo = min(lo, top[l]);
+            hi = max(hi, top[l] + 3);
+        }
+#pragma unroll 1
+        for (int k = 0; k < N1; ++k) {
+            Fix cxa[4][N1];
+            int col;
+            {
+                Fix lx[4];
+                col = X - wx0 - 1 + fix_departure(__double2ll_rn(-fma(st, L.c[k], ux) * dt54), lx);
+#pragma unroll
+                for (int a = 0; a < N1; ++a) {
+                    const Fix g = fix_gauge<N1>(F, k, a, dex[a]);
+#pragma unroll
+                    for (int jx = 0; jx < 4; ++jx) cxa[jx][a] = fix_split(fix_mul(lx[jx], g));
+                }
+            }
+            Fix wg[N1][N1];  // w_(k,l) G_y[l][b]
+#pragma unroll
+            for (int l = 0; l < N1; ++l) {
+                bool big = false;
+                const Fix w = fix_split(fix_population(A.w[(long long)(N1 * k + l) * N + node], scale, big));
+#pragma unroll
+                for (int b = 0; b < N1; ++b) {
+                    const int2 v = s_gy[(N1 * l + b) * NT + tid];
+                    wg[l][b] = fix_split(fix_mul(Fix{v.x, v.y}, w));
+                }
+            }
+#pragma unroll 1
+            for (int y = lo; y <= hi; ++y) {
+                long long vh[N1], vm[N1];
+#pragma unroll
+                for (int b = 0; b < N1; ++b) vh[b] = vm[b] = 0;
+                bool any = false;
+#pragma unroll
+                for (int l = 0; l < N1; ++l) {
+                    const unsigned j = (unsigned)(y - top[l]);
+                    if (j > 3u) continue;
+                    any = true;
+                    const int2 v = s_ly[(4 * l + (int)j) * NT + tid];
+#pragma unroll
+                    for (int b = 0; b < N1; ++b) fix_mad(Fix{v.x, v.y}, wg[l][b].h, wg[l][b].l, vh[b], vm[b]);
+                }
+                if (!any) continue;
+                Fix V[N1];
+#pragma unroll
+                for (int b = 0; b < N1; ++b) V[b] = fix_split(fix_sum_rn(vh[b], vm[b]));
+                const int at = y * ww + col;
+#pragma unroll
+                for (int jx = 0; jx < 4; ++jx)
+#pragma unroll
+                    for (int a = 0; a < N1; ++a)
+#pragma unroll
+                        for (int b = 0; b < N1; ++b) {
+                            long long h = 0, mm = 0;
+                            fix_mad(cxa[jx][a], V[b].h, V[b].l, h, mm);
+                            const int i = (N1 * a + b) * WN + at + jx;
+                            atomic_add64(s_lo + i, s_hi + i, fix_sum_rn(h, mm));
+                        }
+            }
+        }
+    }
+    __syncthreads();
+
+    // the sources' sums into their own frames
+    const double inv_rst = 1.0 / rst;
+    double* out = win + (size_t)blockIdx.x * Q * WN;
+    const float inv_ww = 1.0f / (float)ww;
+    for (int i = tid; i < wn; i += NT) {
+        const int cy = window_row(i, inv_ww), cx = i - cy * ww;
+        const long long s = (long long)wrap_near(wy0 + cy, A.ny) * A.nx + wrap_near(wx0 + cx, A.nx);
+        const double r = (A.in.st[s] - rst) * inv_rst;
+        const double dx = (A.in.ux[s] - rux) * inv_rst, dy = (A.in.uy[s] - ruy) * inv_rst;
+        double h[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const double v = (double)((long long)((unsigned long long)s_hi[q * WN + i] << 32 | s_lo[q * WN + i]));
+            h[q] = v * pow2d(-scale);
+        }
+        double e[N1][N1];  // [k][a] of G(s -> r) - I, by y, then by x
+        double H[Q];
+#pragma unroll
+        for (int b = 0; b < N1; ++b) {
+            const double de = fma(L.c[b], r, dy);
+#pragma unroll
+            for (int l = 0; l < N1; ++l) e[l][b] = gauge_tail<N1>(L.d3[l], L.d2[l][b], L.d1[l][b], de) * de;
+        }
+#pragma unroll
+        for (int a = 0; a < N1; ++a)
+#pragma unroll
+            for (int b = 0; b < N1; ++b) {
+                double v = h[N1 * a + b];
+#pragma unroll
+                for (int l = 0; l < N1; ++l) v = fma(e[l][b], h[N1 * a + l], v);
+                H[N1 * a + b] = v;
+            }
+#pragma unroll
+        for (int a = 0; a < N1; ++a) {
+            const double de = fma(L.c[a], r, dx);
+#pragma unroll
+            for (int k = 0; k < N1; ++k) e[k][a] = gauge_tail<N1>(L.d3[k], L.d2[k][a], L.d1[k][a], de) * de;
+        }
+#pragma unroll
+        for (int a = 0; a < N1; ++a)
+#pragma unroll
+            for (int b = 0; b < N1; ++b) {
+                double v = H[N1 * a + b];
+#pragma unroll
+                for (int k = 0; k < N1; ++k) v = fma(e[k][a], H[N1 * k + b], v);
+                out[(N1 * a + b) * WN + i] = v;
+            }
+    }
+}
+
+// f_bar of every source from the tiles whose windows hold it (an image of it,
+// where the grid is narrower than a window), and its gauge cotangent, from
+//   d g / d u_x [k][l] = sum_a d1[k][a] f[a][l] / s  and so on (k_adjoint_sources_t),
+// through M[k][a] = sum_l f_bar[k][l] f[a][l] and its y-counterpart.
+template <int N1>
+__global__ void __launch_bounds__(128)
+k_adjoint_reduce(AdjArgs A, const double* __restrict__ win, const ScatterTile* __restrict__ tiles) {
+    constexpr int Q = N1 * N1, WN = ADJ_SCATTER_WN;
+    const Lattice& L = c_La[lattice_slot(N1)];
+    const long long src = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (src >= A.N) return;
+    const int JX = (int)(src % A.nx), JY = (int)(src / A.nx);
+    const int tiles_x = (A.nx + 31) / 32, tiles_y = (A.ny + ADJ_TY - 1) / ADJ_TY;
+    double fb[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) fb[q] = 0.0;
+    // tile origins t0 whose window can hold x: x + vlo dt - 31 - 5 <= t0 <= x + vhi dt + 5
+    double vx0 = A.vlo_x[0], vx1 = A.vhi_x[0], vy0 = A.vlo_y[0], vy1 = A.vhi_y[0];
+#pragma unroll
+    for (int i = 1; i < N1; ++i) {
+        vx0 = fmin(vx0, A.vlo_x[i]);
+        vx1 = fmax(vx1, A.vhi_x[i]);
+        vy0 = fmin(vy0, A.vlo_y[i]);
+        vy1 = fmax(vy1, A.vhi_y[i]);
+    }
+    // (a left tile has no window: bounds beyond its 400 nodes are not needed)
+    const int xa = (int)floor(fmax(vx0 * A.dt, -500.0)) - 36, xb = (int)ceil(fmin(vx1 * A.dt, 500.0)) + 5;
+    const int ya = (int)floor(fmax(vy0 * A.dt, -500.0)) - (ADJ_TY + 4), yb = (int)ceil(fmin(vy1 * A.dt, 500.0)) + 5;
+    // images x + m n with a tile origin in [0, n - 1] in reach
+    const int my0 = -(JY + yb) / A.ny - 1, my1 = (A.ny - 1 - JY - ya) / A.ny + 1;
+    const int mx0 = -(JX + xb) / A.nx - 1, mx1 = (A.nx - 1 - JX - xa) / A.nx + 1;
+    for (int my = my0; my <= my1; ++my) {
+        const int y = JY + my * A.ny;
+        const int tya = max(0, (y + ya) / ADJ_TY - 1), tyb = min(tiles_y - 1, (y + yb) / ADJ_TY);
+        for (int ty = tya; y + yb >= 0 && ty <= tyb; ++ty)
+            for (int mx = mx0; mx <= mx1; ++mx) {
+                const int x = JX + mx * A.nx;
+                const int txa = max(0, (x + xa) / 32 - 1), txb = min(tiles_x - 1, (x + xb) / 32);
+                for (int tx = txa; x + xb >= 0 && tx <= txb; ++tx) {
+                    const long long t = (long long)ty * tiles_x + tx;
+                    const ScatterTile w = tiles[t];
+                    const int cx = x - w.x0, cy = y - w.y0;
+                    if (cx < 0 || cx >= w.w || cy < 0 || cy >= w.h) continue;
+                    const double* p = win + (size_t)t * Q * WN + cy * w.w + cx;
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) fb[q] += p[(size_t)q * WN];
+                }
+            }
+    }
+    double f[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        f[q] = A.in.f[(long long)q * A.N + src];
+        A.fbar_in[(long long)q * A.N + src] = fb[q];
+    }
+    double bux = 0.0, buy = 0.0, bst = 0.0;
+#pragma unroll
+    for (int k = 0; k < N1; ++k)
+#pragma unroll
+        for (int a = 0; a < N1; ++a) {
+            double mx = 0.0, my = 0.0;
+#pragma unroll
+            for (int i = 0; i < N1; ++i) {
+                mx = fma(fb[N1 * k + i], f[N1 * a + i], mx);
+                my = fma(fb[N1 * i + k], f[N1 * i + a], my);
+            }
+            const double d = L.d1[k][a];
+            bux = fma(d, mx, bux);
+            buy = fma(d, my, buy);
+            bst = fma(d * L.c[a], mx + my, bst);
+        }
+    const double stj = A.in.st[src], is = 1.0 / stj;
+    A.gbar_in[src] = bux * is;
+    A.gbar_in[A.N + src] = buy * is;
+    // s = sqrt(T / T_L): dL/dT = dL/ds / (2 s T_L)
+    A.gbar_in[2 * A.N + src] = bst * is / (2.0 * stj * A.T_L);
+}
+
+// Phase B of the staged contexts: the scatter, its reduction, and the gather
+// over the tiles the scatter left (usually none: its CTAs then end at once).
+// 256^2: 2.02 ms for the gather alone, 0.37 ms so (scatter 310, reduction 58 us); 4
+// steps forward and back 14.9 -> 8.4 ms.
+cudaError_t launch_adjoint_phase_b_staged(const AdjArgs& A, int n1, double c_max, double* win,
+                                          ScatterTile* tiles, unsigned int* left, int sms,
+                                          cudaStream_t s) {
+    static int s_set[64][2] = {{0}};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    const size_t smem = (size_t)8 * n1 * n1 * ADJ_SCATTER_WN + (size_t)32 * ADJ_TY * 8 * (n1 * n1 + 4 * n1);
+    void (*kern)(AdjArgs, double, double*, ScatterTile*, unsigned int*) =
+        n1 == 3 ? k_adjoint_scatter<3> : k_adjoint_scatter<4>;
+    int& set = s_set[dev][n1 == 3 ? 1 : 0];
+    if ((int)smem > set) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        set = (int)smem;
+    }
+    e = cudaMemsetAsync(left, 0, sizeof(unsigned int), s);
+    if (e != cudaSuccess) return e;
+    const unsigned n_tiles = (unsigned)(((A.nx + 31) / 32) * ((A.ny + ADJ_TY - 1) / ADJ_TY));
+    kern<<<n_tiles, 32 * ADJ_TY, smem, s>>>(A, c_max, win, tiles, left);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const unsigned nb = (unsigned)((A.N + 127) / 128);
+    if (n1 == 3) k_adjoint_reduce<3><<<nb, 128, 0, s>>>(A, win, tiles);
+    else k_adjoint_reduce<4><<<nb, 128, 0, s>>>(A, win, tiles);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const long long all = (A.N + ADJ_GATHER_WARPS - 1) / ADJ_GATHER_WARPS;
+    const unsigned ng = (unsigned)(all < 16 * sms ? all : 16 * sms);
+    if (n1 == 3) k_adjoint_sources_t<3><<<ng, ADJ_GATHER_WARPS * 32, 0, s>>>(A, left);
+    else k_adjoint_sources_t<4><<<ng, ADJ_GATHER_WARPS * 32, 0, s>>>(A, left);
+    return cudaGetLastError();
+}
+
 template <int N1>
 __global__ void k_rho_bar(const double* __restrict__ fbar, double* __restrict__ rbar, long long N) {
     const Lattice& L = c_La[lattice_slot(N1)];
@@ -1513,6 +1901,8 @@ void destroy_adjoint(pond_ctx* ctx) {
     cudaFree(a->org1);
     cudaFree(a->lw1);
     cudaFree(a->redo);
+    cudaFree(a->win);
+    cudaFree(a->tiles);
     cudaFree(a->inv_st);
     cudaFree(a->jvp);
     cudaFree(a->nu_dev);
@@ -1632,7 +2022,10 @@ static pond_status adjoint_step_impl(pond_ctx* ctx, const double* const out_gaug
                 const size_t tiles = ((size_t)(G0.nx + 31) / 32) * (((size_t)G0.ny + 3) / 4);
                 ACK(cudaMalloc(&a->org1, sizeof(int) * 2 * 4 * N), "adjoint alloc");
                 ACK(cudaMalloc(&a->lw1, sizeof(double) * 2 * 4 * 4 * N), "adjoint alloc");
+                const size_t tiles8 = ((size_t)(G0.nx + 31) / 32) * (((size_t)G0.ny + ADJ_TY - 1) / ADJ_TY);
                 ACK(cudaMalloc(&a->redo, sizeof(unsigned int) * (1 + 2 * tiles)), "adjoint alloc");
+                ACK(cudaMalloc(&a->win, sizeof(double) * ctx->L.q * ADJ_SCATTER_WN * tiles8), "adjoint alloc");
+                ACK(cudaMalloc(&a->tiles, sizeof(ScatterTile) * tiles8), "adjoint alloc");
             } else {
                 ACK(cudaMalloc(&a->org, sizeof(int2) * 16 * N), "adjoint alloc");
                 ACK(cudaMalloc(&a->lw, sizeof(double) * 8 * 16 * N), "adjoint alloc");
@@ -1735,9 +2128,10 @@ static pond_status adjoint_step_impl(pond_ctx* ctx, const double* const out_gaug
     }
     ACK(cudaGetLastError(), "adjoint targets");
     if (ctx_staged(ctx)) {
-        const unsigned nbt = (unsigned)((N + ADJ_GATHER_WARPS - 1) / ADJ_GATHER_WARPS);
-        if (ctx->L.n1 == 3) k_adjoint_sources_t<3><<<nbt, ADJ_GATHER_WARPS * 32, 0, s>>>(A);
-        else k_adjoint_sources_t<4><<<nbt, ADJ_GATHER_WARPS * 32, 0, s>>>(A);
+        int sms = 0;
+        ACK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device), "SM count");
+        ACK(launch_adjoint_phase_b_staged(A, ctx->L.n1, ctx->L.c_max, a->win, a->tiles, a->redo, sms, s),
+            "adjoint sources (staged)");
     } else {
         if (ctx->L.n1 == 3) k_adjoint_sources<3><<<nb, ADJ_WARPS * 32, 0, s>>>(A);
         else k_adjoint_sources<4><<<nb, ADJ_WARPS * 32, 0, s>>>(A);

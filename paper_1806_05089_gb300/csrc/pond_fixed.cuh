@@ -88,14 +88,16 @@ __host__ __device__ __forceinline__ Fix fix_split(long long v) {
     return f;
 }
 
-inline LatticeFix make_lattice_fix(const Lattice& L) {
+// (scaled = false: without those factors)
+inline LatticeFix make_lattice_fix(const Lattice& L, bool scaled = true) {
     LatticeFix F{};
     auto fx = [](double v) { return (long long)std::llrint(v * kFixOne); };
     for (int k = 0; k < L.n1; ++k) {
         F.c[k] = fix_split(fx(L.c[k]));
         for (int a = 0; a < L.n1; ++a) {
-            const int s = L.n1 == 4 ? fix_shift<4>(k) - fix_shift<4>(a)
-                                    : fix_shift<3>(k) - fix_shift<3>(a);
+            const int s = !scaled     ? 0
+                          : L.n1 == 4 ? fix_shift<4>(k) - fix_shift<4>(a)
+                                      : fix_shift<3>(k) - fix_shift<3>(a);
             F.d0[k][a] = k == a ? fx(1.0) : 0;
             F.d1[k][a] = fx(std::ldexp(L.d1[k][a], s));
             F.d2[k][a] = fx(std::ldexp(L.d2[k][a], s));
@@ -121,6 +123,11 @@ __device__ __forceinline__ void fix_mad(Fix w, int gh, int gl, long long& h, lon
 // The dot product h 2^64 + m 2^32 of weights and values, in the values' scale.
 __device__ __forceinline__ long long fix_sum(long long h, long long m) {
     return (h << (64 - kFix)) + (m >> (kFix - 32));
+}
+
+// The same, rounded to nearest.
+__device__ __forceinline__ long long fix_sum_rn(long long h, long long m) {
+    return (h << (64 - kFix)) + ((m + (1ll << (kFix - 33))) >> (kFix - 32));
 }
 
 // Product of a weight and v, in v's scale.
