@@ -39,6 +39,9 @@ struct AdjMixedScratch {
     float4* f4 = nullptr;     // [4][N] the input populations as rows f[a][0..n1-1]
     int2* org = nullptr;      // [16][N] stencil origin of (q, t), relative to t
     float* lw = nullptr;      // [16][N][8] cubic weights of (q, t): x 0..3, y 0..3
+    // staged contexts keep them per speed and direction instead
+    int4* org1 = nullptr;     // [2][N]
+    float4* lw1 = nullptr;    // [2][4][N]
     float* inv_st = nullptr;  // [N] 1 / s* at every target
     float* vb = nullptr;      // [16] per-speed velocity bounds of lambda* (k_speed_bounds)
 };
@@ -128,8 +131,11 @@ struct AdjMixedArgs {
     double* beta_bar;
     // per (population, target), written by the target kernel for the gather:
     // stencil origin relative to the target, cubic weights, and 1 / s*
+    // (staged contexts: per speed and direction)
     int2* org;
     float* lw;
+    int4 *org_x, *org_y;     // [N], the speeds' origins in x, y, z, w
+    float4 *lw_x, *lw_y;     // [n1][N]
     float* inv_st;
     int nx, ny;
     long long N;
@@ -445,8 +451,9 @@ __global__ void __launch_bounds__(ADJM_THREADS) k_adjoint_sources_mixed(AdjMixed
 // pair are a product set K x L, since the x-stencil's origin depends on the
 // x-speed alone and the y-stencil's on the y-speed alone.  Each thread walks the union of its
 // source's candidate windows once, evaluates a hit target's rows G_x[k][.]
-// (k in K) and G_y[l][.] (l in L) once, then does each hit's weight and
-// rank-one update.
+// (k in K) and G_y[l][.] (l in L) once, sums the hits of one k over L, and
+// does one rank-one update per k (512^2: 402 us with one per hit and the
+// stencils read per population, 321 us so).
 template <int N1>
 __global__ void __launch_bounds__(ADJM_THREADS, 5)  // 5 CTAs per SM: measured 2 % faster than 4
 k_adjoint_sources_mixed_t(AdjMixedArgs A) {
@@ -483,14 +490,16 @@ k_adjoint_sources_mixed_t(AdjMixedArgs A) {
         int tx = tx0;
         for (int xx = xlo; xx <= xhi; ++xx, tx = (tx + 1 == A.nx) ? 0 : tx + 1) {
             const long long t = row + tx;
+            const int4 ox4 = A.org_x[t], oy4 = A.org_y[t];
+            const int ox[4] = {ox4.x, ox4.y, ox4.z, ox4.w}, oy[4] = {oy4.x, oy4.y, oy4.z, oy4.w};
             int jx[N1], jy[N1];
             unsigned kmask = 0u, lmask = 0u;
 #pragma unroll
             for (int i = 0; i < N1; ++i) {
-                jx[i] = JX - (xx + A.org[(long long)(N1 * i) * A.N + t].x);
-                jy[i] = JY - (yy + A.org[(long long)i * A.N + t].y);
-                kmask |= (jx[i] >= 0 && jx[i] <= 3) ? 1u << i : 0u;
-                lmask |= (jy[i] >= 0 && jy[i] <= 3) ? 1u << i : 0u;
+                jx[i] = JX - (xx + ox[i]);
+                jy[i] = JY - (yy + oy[i]);
+                kmask |= (unsigned)jx[i] <= 3u ? 1u << i : 0u;
+                lmask |= (unsigned)jy[i] <= 3u ? 1u << i : 0u;
             }
             if (!kmask || !lmask) continue;
             const float4 th = A.gstar[t], tl = A.gstar[A.N + t];
@@ -498,40 +507,39 @@ k_adjoint_sources_mixed_t(AdjMixedArgs A) {
             const float r = sdiff(jh.x, jl.x, th.x, tl.x) * inv;
             const float dx = sdiff(jh.y, jl.y, th.y, tl.y) * inv;
             const float dy = sdiff(jh.z, jl.z, th.z, tl.z) * inv;
-            float gx[N1][N1], gy[N1][N1], lxs[N1], lys[N1];
-#pragma unroll
-            for (int k = 0; k < N1; ++k) {
-                lxs[k] = 0.0f;
-                if (!(kmask >> k & 1u)) continue;
-                lxs[k] = A.lw[8 * ((long long)(N1 * k) * A.N + t) + jx[k]];
-#pragma unroll
-                for (int a = 0; a < N1; ++a)
-                    gx[k][a] = gauge_poly<N1>(L.d3[k], L.d2[k][a], L.d1[k][a], a == k ? 1.0f : 0.0f,
-                                              fmaf(L.c[a], r, dx));
-            }
+            // ly_l G_y[l][.] of the hit rows
+            float gy[N1][N1];
 #pragma unroll
             for (int l = 0; l < N1; ++l) {
-                lys[l] = 0.0f;
+#pragma unroll
+                for (int b = 0; b < N1; ++b) gy[l][b] = 0.0f;
                 if (!(lmask >> l & 1u)) continue;
-                lys[l] = A.lw[8 * ((long long)l * A.N + t) + 4 + jy[l]];
+                const float wy = reinterpret_cast<const float*>(A.lw_y + (long long)l * A.N + t)[jy[l]];
 #pragma unroll
                 for (int b = 0; b < N1; ++b)
-                    gy[l][b] = gauge_poly<N1>(L.d3[l], L.d2[l][b], L.d1[l][b], b == l ? 1.0f : 0.0f,
-                                              fmaf(L.c[b], r, dy));
+                    gy[l][b] = wy * gauge_poly<N1>(L.d3[l], L.d2[l][b], L.d1[l][b], b == l ? 1.0f : 0.0f,
+                                                   fmaf(L.c[b], r, dy));
             }
+            // per hit x-speed: u = sum_l w_(k,l) ly_l G_y[l][.], then one rank-one
+            // update with lx_k G_x[k][.]
 #pragma unroll
             for (int k = 0; k < N1; ++k) {
                 if (!(kmask >> k & 1u)) continue;
+                float u[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
                 for (int l = 0; l < N1; ++l) {
                     if (!(lmask >> l & 1u)) continue;
-                    const float coef = A.w[(long long)(N1 * k + l) * A.N + t] * (lxs[k] * lys[l]);
+                    const float w = A.w[(long long)(N1 * k + l) * A.N + t];
 #pragma unroll
-                    for (int a = 0; a < N1; ++a) {
-                        const float cgx = coef * gx[k][a];
+                    for (int b = 0; b < N1; ++b) u[b] = fmaf(w, gy[l][b], u[b]);
+                }
+                const float wx = reinterpret_cast<const float*>(A.lw_x + (long long)k * A.N + t)[jx[k]];
 #pragma unroll
-                        for (int b = 0; b < N1; ++b) fb[N1 * a + b] = fmaf(cgx, gy[l][b], fb[N1 * a + b]);
-                    }
+                for (int a = 0; a < N1; ++a) {
+                    const float cgx = wx * gauge_poly<N1>(L.d3[k], L.d2[k][a], L.d1[k][a],
+                                                          a == k ? 1.0f : 0.0f, fmaf(L.c[a], r, dx));
+#pragma unroll
+                    for (int b = 0; b < N1; ++b) fb[N1 * a + b] = fmaf(cgx, u[b], fb[N1 * a + b]);
                 }
             }
         }
@@ -568,12 +576,13 @@ k_adjoint_sources_mixed_t(AdjMixedArgs A) {
 
 // ---------------------------------------------------------------------------
 // Phase A in the staged form (the FP64 counterpart is k_adjoint_jvp_staged in
-// pond_adjoint.cu): the window of sources a 32 x 4 tile of targets can reach
+// pond_adjoint.cu): the window of sources a 32 x 8 tile of targets can reach
 // is staged once in the tile's reference gauge lambda_r (FP32 rows, the
-// forward step's own staging), and each population's A* and its three
-// tangents come from one pass over its four stencil rows: the rows
-// interpolated with the cubic weights (Fi) and with their derivatives (Fd),
-// the x-map r -> lambda* applied, the y-map after.  The per-node epilogue of
+// forward step's own staging), and the populations' A* and three tangents
+// come from one sweep per x-speed over the rows of the union of its y-stencils
+// (9 rows instead of 4 per population, on packed FP32 pairs; 512^2: 291 -> 228
+// us): the rows interpolated with the cubic weights (Fi) and with their
+// derivatives (Fd), the x-map r -> lambda* applied, the y-map after.  The per-node epilogue of
 // k_adjoint_targets_mixed follows in the same thread (running sums over the
 // populations, the 3 x 3 solve, w, the beta cotangent), so A* and its
 // tangents never leave registers.
@@ -590,7 +599,7 @@ struct StagedAdj32 {
     }
 };
 
-constexpr int ADJM_TY = 4;  // staged phase A tile: 32 x 4 targets
+constexpr int ADJM_TY = 8;  // staged phase A tile: 32 x 8 targets (238 us at 512^2; 32 x 4: 243)
 
 // L_k(c_a + de) - [k == a] in correction form, and L_k'(c_a + de)
 __device__ __forceinline__ void lag_taylor_ef(const LatticeF& L, int k, int a, float de, float& e,
@@ -676,12 +685,13 @@ __device__ __noinline__ void adj_population_direct_mixed(const AdjMixedArgs& A, 
 // beta cotangent.  in: the step's input state; ux_star / uy_star (and
 // A.st_star): lambda* in FP64; wwa x wha: the window capacity.
 template <int N1>
-__global__ void __launch_bounds__(32 * ADJM_TY, 3)  // 3 CTAs per SM: measured 2 % faster than 2
+__global__ void __launch_bounds__(32 * ADJM_TY, 1)  // 12 warps per SM at 168 registers spill: 386 us
 k_adjoint_jvp_staged_mixed(AdjMixedArgs A, StateBuf<float> in, const double* __restrict__ ux_star,
                            const double* __restrict__ uy_star, int wwa, int wha, float c_max) {
     constexpr int TX = 32, NT = TX * ADJM_TY, Q = N1 * N1;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    extern __shared__ __align__(32) unsigned char smem_raw[];
     float4* s_f = reinterpret_cast<float4*>(smem_raw);  // [N1][WN]
+    __shared__ float4 s_ly[N1 * NT], s_dy[N1 * NT];     // y-weights, their derivatives
     __shared__ float s_red[4][NT / 32];
     const LatticeF& L = c_Lam[lattice_slot(N1)];
     const int WN = wwa * wha;
@@ -750,7 +760,28 @@ k_adjoint_jvp_staged_mixed(AdjMixedArgs A, StateBuf<float> in, const double* __r
         float rho = 0.0f, sAf = 0.0f, wf = 0.0f;
         float Px[3] = {0.0f, 0.0f, 0.0f}, Py[3] = {0.0f, 0.0f, 0.0f}, Pt[3] = {0.0f, 0.0f, 0.0f};
         float gF[3] = {0.0f, 0.0f, 0.0f}, gS[3] = {0.0f, 0.0f, 0.0f};
+        // y-stencils of the y-speeds: weights and their derivatives into this
+        // thread's column, and the row that completes each (else -1)
+        int last[N1];
+        int lo = 0x7fffffff, hi = -1;
 #pragma unroll
+        for (int l = 0; l < N1; ++l) {
+            const float fry = -fmaf(st, L.c[l], uy) * dt;
+            const float fly = floorf(fry);
+            float ly[4], dly[4];
+            lagrange4_df(fry - fly + 1.0f, ly, dly);
+            s_ly[l * NT + tid] = make_float4(ly[0], ly[1], ly[2], ly[3]);
+            s_dy[l * NT + tid] = make_float4(dly[0], dly[1], dly[2], dly[3]);
+            reinterpret_cast<int*>(A.org_y + node)[l] = (int)fly - 1;
+            A.lw_y[(long long)l * A.N + node] = make_float4(ly[0], ly[1], ly[2], ly[3]);
+            const int top = Y + (int)fly - 1 - wy0;
+            last[l] = top >= 0 && top + 3 < wh ? top + 3 : -1;
+            if (last[l] >= 0) {
+                lo = min(lo, top);
+                hi = max(hi, top + 3);
+            }
+        }
+#pragma unroll 1
         for (int k = 0; k < N1; ++k) {
             const float ck = L.c[k];
             const float frx = -fmaf(st, ck, ux) * dt;
@@ -758,106 +789,19 @@ k_adjoint_jvp_staged_mixed(AdjMixedArgs A, StateBuf<float> in, const double* __r
             float lx[4], dlx[4];
             lagrange4_df(frx - flx + 1.0f, lx, dlx);
             const int col = X + (int)flx - 1 - wx0;
+            const bool on = col >= 0 && col + 3 < ww;
+            // x-map entries of a = k, k + 1, ... (cyclic)
             float ex[N1], gdx[N1], gdxx[N1];
 #pragma unroll
-            for (int a = 0; a < N1; ++a) {
+            for (int i = 0; i < N1; ++i) {
+                const int a = k + i < N1 ? k + i : k + i - N1;
                 const float de = fmaf(L.c[a], rt, dxt);
-                lag_taylor_ef(L, k, a, de, ex[a], gdx[a]);
-                gdxx[a] = gdx[a] * (L.c[a] + de);
+                lag_taylor_ef(L, k, a, de, ex[i], gdx[i]);
+                gdxx[i] = gdx[i] * (L.c[a] + de);
             }
-#pragma unroll 1
-            for (int l = 0; l < N1; ++l) {
+            auto population = [&](int l, const float (&R)[4]) {
                 const float cl = L.c[l];
-                const float fry = -fmaf(st, cl, uy) * dt;
-                const float fly = floorf(fry);
-                float ly[4], dly[4];
-                lagrange4_df(fry - fly + 1.0f, ly, dly);
-                const int top = Y + (int)fly - 1 - wy0;
-                const int q = N1 * k + l;
-                const long long o = (long long)q * A.N + node;
-                A.org[o] = make_int2((int)flx - 1, (int)fly - 1);
-                float4* pw = reinterpret_cast<float4*>(A.lw + 8 * o);
-                pw[0] = make_float4(lx[0], lx[1], lx[2], lx[3]);
-                pw[1] = make_float4(ly[0], ly[1], ly[2], ly[3]);
-                float R[4];
-                if (col >= 0 && col + 3 < ww && top >= 0 && top + 3 < wh) {
-                    float Z[N1], Zux[N1], Zuy[N1], Zs[N1];
-#pragma unroll
-                    for (int b = 0; b < N1; ++b) Z[b] = Zux[b] = Zuy[b] = Zs[b] = 0.0f;
-#pragma unroll 1
-                    for (int jy = 0; jy < 4; ++jy) {
-                        const float w = jy == 0 ? ly[0] : jy == 1 ? ly[1] : jy == 2 ? ly[2] : ly[3];
-                        const float dw = jy == 0 ? dly[0] : jy == 1 ? dly[1] : jy == 2 ? dly[2] : dly[3];
-                        const float4* src = s_f + (top + jy) * ww + col;
-                        float Fi[N1][N1], Fd[N1][N1];
-#pragma unroll
-                        for (int a = 0; a < N1; ++a)
-#pragma unroll
-                            for (int b = 0; b < N1; ++b) Fi[a][b] = Fd[a][b] = 0.0f;
-#pragma unroll
-                        for (int jx = 0; jx < 4; ++jx) {
-#pragma unroll
-                            for (int a = 0; a < N1; ++a) {
-                                const float4 v = src[(size_t)a * WN + jx];
-                                const float fr[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                                for (int b = 0; b < N1; ++b) {
-                                    Fi[a][b] = fmaf(lx[jx], fr[b], Fi[a][b]);
-                                    Fd[a][b] = fmaf(dlx[jx], fr[b], Fd[a][b]);
-                                }
-                            }
-                        }
-                        // the row's contributions: value, and the tangents
-                        // through the x-weights (Fd), the x-map (gdx) and
-                        // the row weight (dw)
-                        const float wux = -dt * w, wdy = -dt * dw, wi = -w * inv;
-#pragma unroll
-                        for (int b = 0; b < N1; ++b) {
-                            float P = Fi[k][b], P1 = Fd[k][b], Pd = 0.0f, Pdx = 0.0f;
-#pragma unroll
-                            for (int a = 0; a < N1; ++a) {
-                                P = fmaf(ex[a], Fi[a][b], P);
-                                P1 = fmaf(ex[a], Fd[a][b], P1);
-                                Pd = fmaf(gdx[a], Fi[a][b], Pd);
-                                Pdx = fmaf(gdxx[a], Fi[a][b], Pdx);
-                            }
-                            Z[b] = fmaf(w, P, Z[b]);
-                            Zux[b] = fmaf(wux, P1, fmaf(wi, Pd, Zux[b]));
-                            Zuy[b] = fmaf(wdy, P, Zuy[b]);
-                            Zs[b] = fmaf(ck * wux, P1, fmaf(wi, Pdx, fmaf(cl * wdy, P, Zs[b])));
-                        }
-                    }
-                    // the y-map r -> lambda* and its derivatives; its
-                    // identity part exactly
-                    float Al = 0.0f, Axl = 0.0f, Ayl = 0.0f, Asl = 0.0f;
-#pragma unroll
-                    for (int b = 0; b < N1; ++b) {
-                        const bool id = b == l;
-                        Al += id ? Z[b] : 0.0f;
-                        Axl += id ? Zux[b] : 0.0f;
-                        Ayl += id ? Zuy[b] : 0.0f;
-                        Asl += id ? Zs[b] : 0.0f;
-                    }
-                    float Ae = 0.0f, Axe = 0.0f, Aye = 0.0f, Ase = 0.0f, Dy = 0.0f, Ds = 0.0f;
-#pragma unroll
-                    for (int b = 0; b < N1; ++b) {
-                        const float de = fmaf(L.c[b], rt, dyt);
-                        float ey, gdy;
-                        lag_taylor_ef(L, l, b, de, ey, gdy);
-                        Ae = fmaf(ey, Z[b], Ae);
-                        Axe = fmaf(ey, Zux[b], Axe);
-                        Aye = fmaf(ey, Zuy[b], Aye);
-                        Ase = fmaf(ey, Zs[b], Ase);
-                        Dy = fmaf(gdy, Z[b], Dy);
-                        Ds = fmaf(gdy * (L.c[b] + de), Z[b], Ds);
-                    }
-                    R[0] = Al + Ae;
-                    R[1] = Axl + Axe;
-                    R[2] = fmaf(-inv, Dy, Ayl + Aye);
-                    R[3] = fmaf(-inv, Ds, Asl + Ase);
-                } else {
-                    adj_population_direct_mixed<N1>(A, X, Y, k, l, th, tl, st, ux, uy, inv, R);
-                }
+                const long long o = (long long)(N1 * k + l) * A.N + node;
                 const float fb = (float)A.fbar[o];
                 const float mt = fmaf(ck, ck, cl * cl) - 2.0f * T_L;
                 rho += R[0];
@@ -870,6 +814,126 @@ k_adjoint_jvp_staged_mixed(AdjMixedArgs A, StateBuf<float> in, const double* __r
                     Pt[j] = fmaf(mt, R[1 + j], Pt[j]);
                     gF[j] = fmaf(fb, R[1 + j], gF[j]);
                     gS[j] += R[1 + j];
+                }
+            };
+            reinterpret_cast<int*>(A.org_x + node)[k] = (int)flx - 1;
+            A.lw_x[(long long)k * A.N + node] = make_float4(lx[0], lx[1], lx[2], lx[3]);
+#pragma unroll 1
+            for (int l = 0; l < N1; ++l) {
+                int la = last[0];
+#pragma unroll
+                for (int i = 1; i < N1; ++i) la = i == l ? last[i] : la;
+                if (!(on && la >= 0)) {
+                    float R[4];
+                    adj_population_direct_mixed<N1>(A, X, Y, k, l, th, tl, st, ux, uy, inv, R);
+                    population(l, R);
+                }
+            }
+            if (!on) continue;
+            // One sweep over the rows of the union of the y-stencils: a row's
+            // value P and the parts of its u_x- and s-tangents that its row
+            // weight multiplies, U = -dt P1 - P' / s and S = -dt c_k P1 - P'xi / s
+            // (P1: with the x-weights' derivatives; P', P'xi: with the x-map's).
+            // The last four rows' wait in registers; population l is summed
+            // over its rows when the sweep reaches its last one.
+            float2 rP[4][2], rU[4][2], rS[4][2];
+            auto fma2 = [](float w, float2 v, float2 c) { return __ffma2_rn(make_float2(w, w), v, c); };
+#pragma unroll 1
+            for (int y = lo; y <= hi; ++y) {
+                const float4* src = s_f + y * ww + col;
+                float2 P[2], P1[2], Pd[2], Pq[2];
+#pragma unroll
+                for (int i = 0; i < N1; ++i) {
+                    const int a = k + i < N1 ? k + i : k + i - N1;
+                    float2 Fi[2], Fd[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) Fi[h] = Fd[h] = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int jx = 0; jx < 4; ++jx) {
+                        const float4 v = src[a * WN + jx];
+                        const float2 v2[2] = {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            Fi[h] = fma2(lx[jx], v2[h], Fi[h]);
+                            Fd[h] = fma2(dlx[jx], v2[h], Fd[h]);
+                        }
+                    }
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (i == 0) {  // the identity part of the x-map
+                            P[h] = Fi[h];
+                            P1[h] = Fd[h];
+                            Pd[h] = Pq[h] = make_float2(0.f, 0.f);
+                        }
+                        P[h] = fma2(ex[i], Fi[h], P[h]);
+                        P1[h] = fma2(ex[i], Fd[h], P1[h]);
+                        Pd[h] = fma2(gdx[i], Fi[h], Pd[h]);
+                        Pq[h] = fma2(gdxx[i], Fi[h], Pq[h]);
+                    }
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) {
+                        rP[j][h] = rP[j + 1][h];
+                        rU[j][h] = rU[j + 1][h];
+                        rS[j][h] = rS[j + 1][h];
+                    }
+                    const float2 z = make_float2(0.f, 0.f);
+                    rP[3][h] = P[h];
+                    rU[3][h] = fma2(-dt, P1[h], fma2(-inv, Pd[h], z));
+                    rS[3][h] = fma2(-dt * ck, P1[h], fma2(-inv, Pq[h], z));
+                }
+                unsigned todo = 0u;
+#pragma unroll
+                for (int l = 0; l < N1; ++l) todo |= y == last[l] ? 1u << l : 0u;
+                while (todo) {
+                    const int l = __ffs(todo) - 1;
+                    todo &= todo - 1;
+                    const float cl = L.c[l];
+                    const float4 w4 = s_ly[l * NT + tid], d4 = s_dy[l * NT + tid];
+                    const float w[4] = {w4.x, w4.y, w4.z, w4.w}, d[4] = {d4.x, d4.y, d4.z, d4.w};
+                    float2 z2[2], q2[2], u2[2], t2[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        z2[h] = q2[h] = u2[h] = t2[h] = make_float2(0.f, 0.f);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            z2[h] = fma2(w[j], rP[j][h], z2[h]);
+                            q2[h] = fma2(d[j], rP[j][h], q2[h]);
+                            u2[h] = fma2(w[j], rU[j][h], u2[h]);
+                            t2[h] = fma2(w[j], rS[j][h], t2[h]);
+                        }
+                    }
+                    const float Z[4] = {z2[0].x, z2[0].y, z2[1].x, z2[1].y};
+                    const float D[4] = {q2[0].x, q2[0].y, q2[1].x, q2[1].y};
+                    const float U[4] = {u2[0].x, u2[0].y, u2[1].x, u2[1].y};
+                    const float S[4] = {t2[0].x, t2[0].y, t2[1].x, t2[1].y};
+                    // the y-map r -> lambda* and its derivatives; its
+                    // identity part exactly
+                    float Al = 0.0f, Axl = 0.0f, Adl = 0.0f, Asl = 0.0f;
+                    float Ae = 0.0f, Axe = 0.0f, Ade = 0.0f, Ase = 0.0f, Dy = 0.0f, Ds = 0.0f;
+#pragma unroll
+                    for (int b = 0; b < N1; ++b) {
+                        const bool id = b == l;
+                        Al += id ? Z[b] : 0.0f;
+                        Axl += id ? U[b] : 0.0f;
+                        Adl += id ? D[b] : 0.0f;
+                        Asl += id ? S[b] : 0.0f;
+                        const float de = fmaf(L.c[b], rt, dyt);
+                        float ey, gdy;
+                        lag_taylor_ef(L, l, b, de, ey, gdy);
+                        Ae = fmaf(ey, Z[b], Ae);
+                        Axe = fmaf(ey, U[b], Axe);
+                        Ade = fmaf(ey, D[b], Ade);
+                        Ase = fmaf(ey, S[b], Ase);
+                        Dy = fmaf(gdy, Z[b], Dy);
+                        Ds = fmaf(gdy * (L.c[b] + de), Z[b], Ds);
+                    }
+                    const float dtD = -dt * (Adl + Ade);
+                    const float R[4] = {Al + Ae, Axl + Axe, fmaf(-inv, Dy, dtD),
+                                        fmaf(-inv, Ds, fmaf(cl, dtD, Asl + Ase))};
+                    population(l, R);
                 }
             }
         }
@@ -964,6 +1028,8 @@ void destroy_adjoint_mixed(pond_ctx* ctx) {
     cudaFree(a->f4);
     cudaFree(a->org);
     cudaFree(a->lw);
+    cudaFree(a->org1);
+    cudaFree(a->lw1);
     cudaFree(a->inv_st);
     cudaFree(a->vb);
     delete a;
@@ -994,8 +1060,13 @@ cudaError_t adjoint_step_mixed(pond_ctx* ctx, const double* const out_gauge[3],
         if ((e = cudaMalloc(&a->iters, sizeof(int32_t) * N)) != cudaSuccess) return e;
         if ((e = cudaMalloc(&a->stats, sizeof(DevStats))) != cudaSuccess) return e;
         if ((e = cudaMalloc(&a->f4, sizeof(float4) * 4 * N)) != cudaSuccess) return e;
-        if ((e = cudaMalloc(&a->org, sizeof(int2) * 16 * N)) != cudaSuccess) return e;
-        if ((e = cudaMalloc(&a->lw, sizeof(float) * 8 * 16 * N)) != cudaSuccess) return e;
+        if (ctx_staged(ctx)) {
+            if ((e = cudaMalloc(&a->org1, sizeof(int4) * 2 * N)) != cudaSuccess) return e;
+            if ((e = cudaMalloc(&a->lw1, sizeof(float4) * 2 * 4 * N)) != cudaSuccess) return e;
+        } else {
+            if ((e = cudaMalloc(&a->org, sizeof(int2) * 16 * N)) != cudaSuccess) return e;
+            if ((e = cudaMalloc(&a->lw, sizeof(float) * 8 * 16 * N)) != cudaSuccess) return e;
+        }
         if ((e = cudaMalloc(&a->inv_st, sizeof(float) * N)) != cudaSuccess) return e;
         if ((e = cudaMalloc(&a->vb, sizeof(float) * 16)) != cudaSuccess) return e;
     }
@@ -1044,6 +1115,10 @@ cudaError_t adjoint_step_mixed(pond_ctx* ctx, const double* const out_gauge[3],
     A.beta_bar = beta_bar_dev;
     A.org = a->org;
     A.lw = a->lw;
+    A.org_x = a->org1;
+    A.org_y = a->org1 ? a->org1 + N : nullptr;
+    A.lw_x = a->lw1;
+    A.lw_y = a->lw1 ? a->lw1 + 4 * N : nullptr;
     A.inv_st = a->inv_st;
     A.nx = G.nx;
     A.ny = G.ny;
