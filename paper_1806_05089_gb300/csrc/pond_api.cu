@@ -139,7 +139,7 @@ pond_status update_window(pond_ctx* ctx) {
     if (!w.staged)
         CK(mixed_prepare(w.ty, w.pair != 0, w.n1, smem, &per_sm), "mixed kernel set-up");
     else if (mixed(ctx))
-        CK(staged_prepare_mixed(w.ty, w.n1, smem, &per_sm), "staged kernel set-up");
+        CK(staged_prepare_mixed(&w, ex, ey, ctx->n_tiles, sms, &per_sm), "staged kernel set-up");
     else
         CK(staged_prepare_fp64(&w, ex, ey, ctx->n_tiles, sms, &per_sm), "staged kernel set-up");
     if (per_sm < 1) return fail(ctx, POND_ERR_CUDA, "tile kernel does not fit on an SM");

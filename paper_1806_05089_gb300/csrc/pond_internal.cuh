@@ -182,8 +182,9 @@ struct TileWindow {
     int n1;           // speeds per dimension of the lattice (4 or 3)
     int staged;       // 1: the reference-gauge staged kernel
     int real_bytes;   // 8 (FP64 form) or 4 (mixed form)
-    // the FP64 form's fixed-point kernel: its CTA's part of the tile, threads
-    // per node and staged window
+    // the FP64 form's fixed-point kernel, and the mixed form where it runs by
+    // parts (else fx = 0): a CTA's part of the tile, threads per node and
+    // staged window
     int fx, fy, fks;
     int fww, fwh;
     // nodes of the two windows, when they are set by capacity and the sides
@@ -220,12 +221,14 @@ cudaError_t launch_step_staged_mixed(const StateBuf<float>& in, const StateBuf<f
                                      int64_t plane, unsigned int* work_counter,
                                      const TileWindow& win, int persistent_ctas, const Lattice& L,
                                      const StepParams& P, cudaStream_t s);
-// (FP64: completes the window with the fixed-point kernel's shape and staged
-// window, for velocity spreads that need ex x ey extra nodes, by the number of
-// 32 x ty tiles a step has)
+// (Both complete the window, for velocity spreads that need ex x ey extra nodes,
+// by the number of 32 x ty tiles a step has: the FP64 form with the fixed-point
+// kernel's shape and staged window, the mixed form with a part of a tile and
+// its window where the tiles do not fill the chip.)
 cudaError_t staged_prepare_fp64(TileWindow* win, int ex, int ey, int64_t n_tiles, int sms,
                                 int* ctas_per_sm);
-cudaError_t staged_prepare_mixed(int ty, int n1, size_t smem, int* ctas_per_sm);
+cudaError_t staged_prepare_mixed(TileWindow* win, int ex, int ey, int64_t n_tiles, int sms,
+                                 int* ctas_per_sm);
 // Extra window extent, in nodes, that one step's departures need for a
 // particle-speed spread `span`: ceil(span * dt + pad), bounded by 65536 so
 // that an absurd spread (a finite but huge temperature or velocity, whose

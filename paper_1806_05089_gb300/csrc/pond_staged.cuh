@@ -259,19 +259,26 @@ __device__ __forceinline__ void stage_window(const StateBuf<typename Tr::Real>& 
     }
 }
 
-template <class Tr, int TX, int TY, int N1>
-__global__ void __launch_bounds__(TX* TY, Tr::template min_blocks<TX * TY>())
+// KS = 1: a thread per node of the TX x TY tile.  KS = 2 or 4 (mixed form, small
+// grids): a CTA takes a part of TXS = 32 / KS columns with KS lanes per node, lane
+// `part` sweeping the x-speeds k = part, part + KS, ..; 32 / KS >= 8 nodes stand
+// side by side, so the 16-byte reads of a quarter warp stay contiguous.  The same
+// sums in the same order (over l per x-speed, then over the x-speeds): a grid's
+// result does not depend on KS.
+template <class Tr, int TX, int TY, int N1, int KS = 1, int TXS = TX>
+__global__ void __launch_bounds__(TXS* TY* KS, Tr::template min_blocks<TXS * TY * KS>())
 k_step_staged(StagedArgs<typename Tr::Real> A) {
     using Real = typename Tr::Real;
     using Real4 = typename Tr::Real4;
-    constexpr int NT = TX * TY;
+    constexpr int NN = TXS * TY, NT = NN * KS, SUB = TX / TXS;
     constexpr unsigned FULL = 0xffffffffu;
-    static_assert(TX == 32, "a warp is one tile row");
+    static_assert(TX == 32 && (KS == 1 ? TXS == 32 : Tr::kPacked && TXS * KS == 32 && !Tr::kEyTable),
+                  "a warp is one tile row, or quarter warps are");
     extern __shared__ __align__(32) unsigned char smem_raw[];
     const int WN = Tr::kRedo ? A.wn : A.ww * A.wh;
     Real4* s_f = reinterpret_cast<Real4*>(smem_raw);              // [N1][WN]: row a of g
-    Real* s_acc = reinterpret_cast<Real*>(s_f + (size_t)N1 * WN);  // [Q][NT]
-    Real* s_ey = s_acc + (size_t)N1 * N1 * NT;  // [Q][NT] Ey[l][b] of the pass (kEyTable)
+    Real* s_acc = reinterpret_cast<Real*>(s_f + (size_t)N1 * WN);  // [Q][NN]
+    Real* s_ey = s_acc + (size_t)N1 * N1 * NN;  // [Q][NT] Ey[l][b] of the pass (kEyTable)
     __shared__ float s_red[4][NT / 32];
     __shared__ long long s_item;
     __shared__ unsigned long long s_passes, s_nc, s_np, s_fb;
@@ -285,7 +292,9 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
         s_fb = 0ull;
         s_max = 0u;
     }
-    const int lxi = tid % TX, lyi = tid / TX;
+    const int lane = tid & 31, part = lane / (32 / KS);
+    const int n = tid / 32 * (32 / KS) + lane % (32 / KS);  // node of the CTA
+    const int lxi = n % TXS, lyi = n / TXS;
     const Real dt = (Real)A.P.dt;
     const unsigned long long t_begin = (A.work_counter && tid == 0) ? pond_globaltimer() : 0ull;
 
@@ -308,7 +317,9 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
             __syncthreads();
             item = s_item;
         }
-        if (item >= A.n_tiles) break;
+        if (item >= A.n_tiles * SUB) break;
+        const int sub = (int)(item % SUB);
+        item /= SUB;
 
         int g = 0;
         if (A.n_grids > 1) {
@@ -324,8 +335,12 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
         // tiles cover the grid's interior rectangle (the whole grid unless a
         // domain decomposition narrowed it to the part inside its halo)
         const int tiles_x = (G.iw + TX - 1) / TX;
-        const int tx0 = G.ix0 + (int)(t % tiles_x) * TX;
+        const int ltx0 = G.ix0 + (int)(t % tiles_x) * TX, tx0 = ltx0 + sub * TXS;
         const int ty0 = G.iy0 + (int)(t / tiles_x) * TY;
+        if (SUB > 1 && tx0 >= G.ix0 + G.iw) {  // nothing of a ragged tile
+            if (!A.work_counter) break;
+            continue;
+        }
         const int X = tx0 + lxi, Y = ty0 + lyi;
         bool valid = X < G.ix0 + G.iw && Y < G.iy0 + G.ih;
         if (redo)  // only the part of the tile that was left over
@@ -338,7 +353,7 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
         // the interior), so the staged sources' gauges differ from lambda_r by
         // at most about half the window
         const long long rnode = base + (long long)min(ty0 + TY / 2, G.iy0 + G.ih - 1) * G.nx +
-                                min(tx0 + TX / 2, G.ix0 + G.iw - 1);
+                                min(ltx0 + TX / 2, G.ix0 + G.iw - 1);
         const double rux = A.in.ux[rnode], ruy = A.in.uy[rnode], rst = A.in.st[rnode];
 
         PassGauge pg;
@@ -372,7 +387,7 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
         const float bxl = fminf(fmaxf(vxlo, -1.0e6f), 1.0e6f), bxh = fminf(fmaxf(vxhi, -1.0e6f), 1.0e6f);
         const float byl = fminf(fmaxf(vylo, -1.0e6f), 1.0e6f), byh = fminf(fmaxf(vyhi, -1.0e6f), 1.0e6f);
         const int wx0 = (int)floorf((float)tx0 - bxh * fdt - m) - 1;
-        const int wx1 = (int)floorf((float)(tx0 + TX - 1) - bxl * fdt + m) + 2;
+        const int wx1 = (int)floorf((float)(tx0 + TXS - 1) - bxl * fdt + m) + 2;
         const int wy0 = (int)floorf((float)ty0 - byh * fdt - m) - 1;
         const int wy1 = (int)floorf((float)(ty0 + TY - 1) - byl * fdt + m) + 2;
         // a tile whose bounds are not finite (NaN gauge) stages a 1 x 1 window
@@ -437,14 +452,16 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
             // rolled, that term is formed exactly as sum_a [a == k] Fi[a][b]
             constexpr int KU = Tr::kUnrollK ? N1 : 1;
 #pragma unroll KU
-            for (int k = 0; k < N1; ++k) {
+            for (int k0 = 0; k0 < N1; k0 += KS) {
+                const int k = KS == 1 ? k0 : min(k0 + part, N1 - 1);
+                const bool mine = KS == 1 || k0 + part < N1;  // D2Q9: a lane idles
                 const Real ck = (Real)L.c[k];
                 Real fx;
                 Real lx[4];
                 Tr::departure(-fma(stf, ck, uxf) * dt, fx, lx);
                 const bool xnear = fabs(fx) < (Real)1.0e6;
                 const int col = xnear ? X - wx0 + (int)fx - 1 : -1;
-                const bool colok = work && xnear && col >= 0 && col + 3 < ww;
+                const bool colok = work && mine && xnear && col >= 0 && col + 3 < ww;
                 Real ext[N1], ik[N1];
 #pragma unroll
                 for (int a = 0; a < N1; ++a) {
@@ -548,7 +565,19 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
                                 Fi2[a][1] = __ffma2_rn(w2, make_float2(v.z, v.w), Fi2[a][1]);
                             }
                         }
-                        float2 P2[2] = {Fi2[k][0], Fi2[k][1]};
+                        float2 P2[2];
+                        if constexpr (KS == 1) {
+                            P2[0] = Fi2[k][0];
+                            P2[1] = Fi2[k][1];
+                        } else {
+                            P2[0] = Fi2[0][0];
+                            P2[1] = Fi2[0][1];
+#pragma unroll
+                            for (int a = 1; a < N1; ++a) {
+                                P2[0] = a == k ? Fi2[a][0] : P2[0];
+                                P2[1] = a == k ? Fi2[a][1] : P2[1];
+                            }
+                        }
 #pragma unroll
                         for (int a = 0; a < N1; ++a) {
                             const float2 e2 = make_float2(ext[a], ext[a]);
@@ -609,7 +638,9 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
                         for (int b = 0; b < N1; ++b) Z[l][b] = z4[b];
                     }
                 }
-                if (work) {
+                // sums over l of f, c_l f and |c|^2 f, then over the x-speeds in order
+                Real a0 = 0, a2 = 0, a3 = 0;
+                if (work && mine) {
 #pragma unroll
                     for (int l = 0; l < N1; ++l) {
                         Real acc = (Real)0;  // stencils off the window: below
@@ -630,14 +661,27 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
                         } else {
                             offwin |= 1u << (N1 * k + l);
                         }
-                        s_acc[(N1 * k + l) * NT + tid] = acc;
+                        s_acc[(N1 * k + l) * NN + n] = acc;
                         const Real cl = (Real)L.c[l];
-                        m0 += acc;
-                        m1 = fma(ck, acc, m1);
-                        m2 = fma(cl, acc, m2);
-                        m3 = fma(fma(ck, ck, cl * cl), acc, m3);
+                        a0 += acc;
+                        a2 = fma(cl, acc, a2);
+                        a3 = fma(fma(ck, ck, cl * cl), acc, a3);
                     }
                 }
+#pragma unroll
+                for (int i = 0; i < KS; ++i) {
+                    if (k0 + i >= N1) break;
+                    const int from = i * (32 / KS) + lane % (32 / KS);
+                    const Real b0 = KS == 1 ? a0 : __shfl_sync(FULL, a0, from);
+                    m0 += b0;
+                    m1 = fma(KS == 1 ? ck : (Real)L.c[k0 + i], b0, m1);
+                    m2 += KS == 1 ? a2 : __shfl_sync(FULL, a2, from);
+                    m3 += KS == 1 ? a3 : __shfl_sync(FULL, a3, from);
+                }
+            }
+            if constexpr (KS > 1) {
+#pragma unroll
+                for (int o = 32 / KS; o < 32; o <<= 1) offwin |= __shfl_xor_sync(FULL, offwin, o);
             }
             // populations whose stencil leaves the staged window, from
             // global memory (outside the sweep, so the sweep keeps its
@@ -647,8 +691,8 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
                 offwin &= offwin - 1;
                 const int k = q / N1, l = q - N1 * k;
                 const Real acc = staged_fallback<Tr, N1>(A, G, base, X, Y, k, l, pg.ux, pg.uy, pg.st);
-                ++fallbacks;
-                s_acc[q * NT + tid] = acc;
+                if (part == 0) ++fallbacks;
+                s_acc[q * NN + n] = acc;
                 const Real ck = (Real)L.c[k], cl = (Real)L.c[l];
                 m0 += acc;
                 m1 = fma(ck, acc, m1);
@@ -657,9 +701,11 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
             }
             if (work) done = Tr::update(A.P, pg, m0, m1, m2, m3);
         }
+        __syncwarp();  // the lanes of a node have stored its populations
         unsigned int passes = 0u;
-        if (valid && POND_INDEX_OK(node >= base && node < base + (long long)G.nx * G.ny, A.stats)) {
-            Tr::template finish<N1>(A, s_acc, NT, tid, node, pg);
+        if (part == 0 && valid &&
+            POND_INDEX_OK(node >= base && node < base + (long long)G.nx * G.ny, A.stats)) {
+            Tr::template finish<N1>(A, s_acc, NN, n, node, pg);
             if (A.iters) A.iters[node] = pg.pass;
             passes = (unsigned int)pg.pass;
             if (pg.flag & 1u) atomicAdd(&s_nc, 1ull);

@@ -1069,34 +1069,79 @@ struct StagedFP32 {
     }
 };
 
+// The kernel of a tile of ty rows: whole, or by parts with ks lanes per node.
 template <int TY, int N1>
-static cudaError_t staged32_shape(size_t smem, int* per_sm, int* s_set) {
-    void (*kern)(StagedArgs<float>) = k_step_staged<StagedFP32, 32, TY, N1>;
-    if ((int)smem > *s_set) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        *s_set = (int)smem;
-    }
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, 32 * TY, smem);
+static void (*staged32_kernel(int ks))(StagedArgs<float>) {
+    if (ks == 4) return k_step_staged<StagedFP32, 32, TY, N1, 4, 8>;
+    if (ks == 2) return k_step_staged<StagedFP32, 32, TY, N1, 2, 16>;
+    return k_step_staged<StagedFP32, 32, TY, N1>;
+}
+static void (*staged32_kernel(int ty, int n1, int ks))(StagedArgs<float>) {
+    if (n1 == 3)
+        return ty == 4 ? staged32_kernel<4, 3>(ks) : ty == 8 ? staged32_kernel<8, 3>(ks) : staged32_kernel<16, 3>(ks);
+    return ty == 4 ? staged32_kernel<4, 4>(ks) : ty == 8 ? staged32_kernel<8, 4>(ks) : staged32_kernel<16, 4>(ks);
 }
 
-cudaError_t staged_prepare_mixed(int ty, int n1, size_t smem, int* ctas_per_sm) {
-    static int s_set[64][6] = {{0}};
+// Lanes per node by the warps a step has (n1 x-speeds; a whole tile's warp is
+// one row).  A warp's chain of passes and rows is what a small grid waits for:
+// with 8 warps on every SM or fewer the issue slots stand idle, and splitting
+// the chain over lanes is worth the sources that neighbouring parts then stage
+// twice.  Measured, supersonic field, us per step with 1 / 2 / 4 lanes (8-row
+// tiles, 152 SMs):
+//              tiles    D2Q16                D2Q9
+//     96^2        36    51.0 / 33.0 / 24.4   33.7 / 26.7 / 20.7
+//    128^2        64    49.3 / 31.9 / 35.0   32.4 / 25.8 / 27.0
+//    193x160     140    49.3 / 47.3 / 62.5   29.8 / 32.9 / 48.3
+//    256x192     192    72.5 / 80.6 / 85.6   41.2 / 50.4 / 66.1
+// so four lanes while those fit on 8 warps per SM, two while they fit on 8
+// (D2Q9) or 16 (D2Q16, whose longer chain is worth more), else one.
+static int staged32_lanes(int n1, int64_t warps, int sms) {
+    if (4 * warps <= 8 * (int64_t)sms) return 4;
+    if (2 * warps <= (n1 == 4 ? 16 : 8) * (int64_t)sms) return 2;
+    return 1;
+}
+
+static size_t staged32_smem(const TileWindow& w) {
+    return w.fx ? staged_smem_bytes(w.n1, w.fww, w.fwh, w.fx * w.fy, sizeof(float))
+                : staged_smem_bytes(w.n1, w.ww, w.wh, w.tx * w.ty, sizeof(float));
+}
+
+cudaError_t staged_prepare_mixed(TileWindow* win, int ex, int ey, int64_t n_tiles, int sms,
+                                 int* ctas_per_sm) {
+    // the attribute is per function and device: only ever raise it, so that
+    // every live context's window stays launchable
+    static int s_set[64][18] = {{0}};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    const int t = ty == 4 ? 0 : ty == 8 ? 1 : ty == 16 ? 2 : -1;
+    const int ty = win->ty, t = ty == 4 ? 0 : ty == 8 ? 1 : ty == 16 ? 2 : -1;
     if (t < 0) return cudaErrorInvalidValue;
-    int* set = &s_set[dev][(n1 == 3 ? 3 : 0) + t];
-    if (n1 == 3) {
-        if (ty == 4) return staged32_shape<4, 3>(smem, ctas_per_sm, set);
-        if (ty == 8) return staged32_shape<8, 3>(smem, ctas_per_sm, set);
-        return staged32_shape<16, 3>(smem, ctas_per_sm, set);
+    for (int ks = staged32_lanes(win->n1, n_tiles * ty, sms);; ks /= 2) {
+        win->fx = win->fy = win->fks = win->fww = win->fwh = 0;
+        if (ks > 1) {
+            win->fx = 32 / ks;
+            win->fy = ty;
+            win->fks = ks;
+            win->fww = win->fx + ex;
+            win->fwh = ty + ey;
+            while (staged32_smem(*win) > 220 * 1024) {
+                if (win->fww - win->fx >= win->fwh - ty) --win->fww; else --win->fwh;
+            }
+        }
+        const int smem = (int)staged32_smem(*win);
+        int* set = &s_set[dev][6 * (ks / 2) + (win->n1 == 3 ? 3 : 0) + t];
+        void (*kern)(StagedArgs<float>) = staged32_kernel(ty, win->n1, ks);
+        if (smem > *set) {
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (e != cudaSuccess) return e;
+            *set = smem;
+        }
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, kern, 32 * ty, smem);
+        // parts whose wide windows do not let them all reside at once would
+        // run one after the other: fewer, larger ones then
+        if (e != cudaSuccess || ks == 1 || n_tiles * ks <= (int64_t)*ctas_per_sm * sms) return e;
     }
-    if (ty == 4) return staged32_shape<4, 4>(smem, ctas_per_sm, set);
-    if (ty == 8) return staged32_shape<8, 4>(smem, ctas_per_sm, set);
-    return staged32_shape<16, 4>(smem, ctas_per_sm, set);
 }
 
 cudaError_t launch_step_staged_mixed(const StateBuf<float>& in, const StateBuf<float>& out,
@@ -1119,33 +1164,22 @@ cudaError_t launch_step_staged_mixed(const StateBuf<float>& in, const StateBuf<f
     A.n_tiles = n_tiles;
     A.plane = plane;
     A.work_counter = work_counter;
-    A.ww = win.ww;
-    A.wh = win.wh;
+    const bool parts = win.fx != 0;
+    A.ww = parts ? win.fww : win.ww;
+    A.wh = parts ? win.fwh : win.wh;
     A.c_max = L.c_max;
     A.margin = 1.0f;
     A.P = P;
-    const size_t smem = staged_smem_bytes(L.n1, win.ww, win.wh, 32 * win.ty, sizeof(float));
+    const int64_t ctas = n_tiles * (parts ? win.tx / win.fx : 1);
     unsigned int nb;
     if (work_counter) {
         cudaError_t e = cudaMemsetAsync(work_counter, 0, sizeof(unsigned int), s);
         if (e != cudaSuccess) return e;
-        nb = (unsigned int)(persistent_ctas < n_tiles ? persistent_ctas : n_tiles);
+        nb = (unsigned int)(persistent_ctas < ctas ? persistent_ctas : ctas);
     } else {
-        nb = (unsigned int)n_tiles;
+        nb = (unsigned int)ctas;
     }
-    if (L.n1 == 3) {
-        switch (win.ty) {
-            case 4: k_step_staged<StagedFP32, 32, 4, 3><<<nb, 128, smem, s>>>(A); break;
-            case 8: k_step_staged<StagedFP32, 32, 8, 3><<<nb, 256, smem, s>>>(A); break;
-            default: k_step_staged<StagedFP32, 32, 16, 3><<<nb, 512, smem, s>>>(A); break;
-        }
-    } else {
-        switch (win.ty) {
-            case 4: k_step_staged<StagedFP32, 32, 4, 4><<<nb, 128, smem, s>>>(A); break;
-            case 8: k_step_staged<StagedFP32, 32, 8, 4><<<nb, 256, smem, s>>>(A); break;
-            default: k_step_staged<StagedFP32, 32, 16, 4><<<nb, 512, smem, s>>>(A); break;
-        }
-    }
+    staged32_kernel(win.ty, L.n1, parts ? win.fks : 1)<<<nb, 32 * win.ty, staged32_smem(win), s>>>(A);
     return cudaGetLastError();
 }
 

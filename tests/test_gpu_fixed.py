@@ -1,6 +1,7 @@
-"""GPU tests of the fixed-point form of the FP64 staged step: the sizes at a
-tile's edges, tiles inside and outside its range of magnitudes and gauge
-spreads in one grid, and its scale.
+"""GPU tests of the forms of the staged step: the fixed-point form of FP64 at
+the sizes of a tile's edges, with tiles inside and outside its range of
+magnitudes and gauge spreads in one grid, and its scale; the mixed form with
+one, two and four lanes per node.
 
 Tolerances: 1e-12 with fixed passes against the oracle, as the other FP64
 parity tests.  The step is homogeneous in the populations and every scale of
@@ -153,3 +154,23 @@ def test_adjoint_step_matches_the_direct_kernels(name, nx, ny, hot, lattice):
             got.append([a.cpu().numpy() for a in out] + [np.array(nu)])
     for a, b in zip(*got):
         assert np.abs(a - b).max() <= 1e-9 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("lattice", [pond.POND_D2Q16, pond.POND_D2Q9])
+@pytest.mark.parametrize("tile_rows,nx,ny", [(8, 31, 7), (8, 70, 45), (8, 161, 100), (4, 97, 65), (16, 130, 90)])
+def test_mixed_lanes_change_no_bit(tile_rows, nx, ny, lattice):
+    """A small grid by itself runs with two or four lanes per node; as the first
+    grid of a batch that fills the chip it runs with one."""
+    T_L = 1.0 / 3.0 if lattice == pond.POND_D2Q9 else 1.0
+    small, large = field("shear", nx, ny, T_L), field("plain", 512, 512, T_L)
+    out = []
+    for grids in ([small], [small, large]):
+        with pond.Sim([g.shape[1] for g in grids], [g.shape[0] for g in grids], pond.POND_FP32_MIXED,
+                      lattice=lattice, T_ref=T_L, tile_rows=tile_rows) as s:
+            for i, g in enumerate(grids):
+                s.set_state(g.rho, g.ux, g.uy, g.T, grid=i)
+            assert s.step(3)["halo_fallback"] == 0
+            out.append(s.state())
+    a, b = out
+    for name in ("f", "ux", "uy", "T"):
+        assert np.array_equal(getattr(a, name), getattr(b, name)), name
