@@ -222,6 +222,8 @@ __device__ __forceinline__ float fix_offset(long long r, long long dx, long long
 // words in s_l, row a at [a * WN + i].  Two planes, so that a quarter warp's
 // 16-byte reads are contiguous.  Returns whether every value this thread
 // staged is in range.
+constexpr int kFixBadSource = (int)0x80000000;  // no staged high word is this
+
 template <int N1, bool WIDE>
 __device__ __forceinline__ bool stage_window_fixed(const StateBuf<double>& in, long long plane,
                                                    const GridDesc& G, long long base, int wx0,
@@ -310,10 +312,59 @@ __device__ __forceinline__ bool stage_window_fixed(const StateBuf<double>& in, l
                 dh[(size_t)k * WN * 4 + 3] = dl[(size_t)k * WN * 4 + 3] = 0;
             }
         }
-        // |g| < R / 4, and the node's largest >= R / 128
-        ok = ok && !big && top < (1 << (kFix - 2 - 32)) && top >= (1 << (kFix - 7 - 32));
+        // |g| < R / 4, and the node's largest >= R / 128; else the source is marked
+        if (big || !(top < (1 << (kFix - 2 - 32)) && top >= (1 << (kFix - 7 - 32)))) {
+            ok = false;
+            s_h[i].x = kFixBadSource;
+        }
     }
     return ok;
+}
+
+// The 8-column groups of a CTA's TXS columns whose own window -- the one a CTA of
+// that group alone stages -- holds a source out of range (kFixBadSource in the
+// staged window at wx0, wy0).  Every thread of the CTA calls it, with its node's
+// velocity and largest thermal speed where `valid`; s_bad is zero on entry.
+template <int TXS, int TYS, int NT>
+__device__ __noinline__ unsigned fixed_bad_groups(const int4* s_h, int wx0, int wy0, int ww, int wh,
+                                                  int tx0, int ty0, float m, float fdt, bool valid,
+                                                  float ux, float uy, float sp, int n,
+                                                  unsigned* s_bad) {
+    constexpr int NG = TXS / 8;
+    __shared__ int s_v[NG][4];  // xlo, xhi, ylo, yhi of a group's nodes, as ordered integers
+    const int tid = threadIdx.x;
+    auto key = [](float v) {
+        const int i = __float_as_int(v);
+        return i >= 0 ? i : i ^ 0x7fffffff;
+    };
+    auto val = [](int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); };
+    if (tid < NG) {
+        s_v[tid][0] = s_v[tid][2] = key(3.0e38f);
+        s_v[tid][1] = s_v[tid][3] = key(-3.0e38f);
+    }
+    __syncthreads();
+    if (valid) {
+        const int g = n % TXS / 8;
+        atomicMin(&s_v[g][0], key(ux - sp));
+        atomicMax(&s_v[g][1], key(ux + sp));
+        atomicMin(&s_v[g][2], key(uy - sp));
+        atomicMax(&s_v[g][3], key(uy + sp));
+    }
+    __syncthreads();
+    for (int i = tid; i < ww * wh; i += NT) {
+        if (s_h[i].x != kFixBadSource) continue;
+        const int x = wx0 + i % ww, y = wy0 + i / ww;
+        for (int g = 0; g < NG; ++g) {
+            const int gx = tx0 + 8 * g;
+            if (x >= (int)floorf((float)gx - val(s_v[g][1]) * fdt - m) - 1 &&
+                x <= (int)floorf((float)(gx + 7) - val(s_v[g][0]) * fdt + m) + 2 &&
+                y >= (int)floorf((float)ty0 - val(s_v[g][3]) * fdt - m) - 1 &&
+                y <= (int)floorf((float)(ty0 + TYS - 1) - val(s_v[g][2]) * fdt + m) + 2)
+                atomicOr(s_bad, 1u << g);
+        }
+    }
+    __syncthreads();
+    return *s_bad;
 }
 
 // The step with its contractions in fixed point: k_step_staged's tile, window,
@@ -328,14 +379,16 @@ __device__ __forceinline__ bool stage_window_fixed(const StateBuf<double>& in, l
 // = part and computing the y-stencil and y-map row l = part; eight nodes stand
 // side by side in a quarter warp, whose 16-byte reads are then contiguous.
 // The gauge update runs in all lanes of a node.  A pass's populations (64-bit
-// integers) wait in the output planes for the closing re-gauge.  Tiles out of
-// range go to A.redo_list.
+// integers) wait in the output planes for the closing re-gauge.  What is out of
+// range goes to A.redo_list, by groups of 8 columns whose nodes and window decide
+// for themselves: which nodes the FP64 form computes does not depend on the shape
+// either, and a steep spot takes 8 columns with it, not a tile.
 template <class Tr, int LTX, int LTY, int TXS, int TYS, int KS, int N1, int MINB>
 __global__ void __launch_bounds__(TXS* TYS* KS, MINB) k_step_fixed(StagedArgs<double> A) {
     constexpr int NN = TXS * TYS, NT = NN * KS, Q = N1 * N1;
-    constexpr int SUBX = LTX / TXS, SUB = SUBX * (LTY / TYS);
+    constexpr int SUB = LTX / TXS, NG = TXS / 8;
     constexpr unsigned FULL = 0xffffffffu;
-    static_assert(NT % 32 == 0 && (KS == 1 || KS == 4) && LTX % TXS == 0 && LTY % TYS == 0,
+    static_assert(NT % 32 == 0 && (KS == 1 || KS == 4) && LTX % TXS == 0 && LTY == TYS && TXS % 8 == 0,
                   "whole warps, the lanes of a node in one");
     extern __shared__ __align__(32) unsigned char smem_raw[];
     const int WN = A.wn;
@@ -347,7 +400,7 @@ __global__ void __launch_bounds__(TXS* TYS* KS, MINB) k_step_fixed(StagedArgs<do
     __shared__ float s_red[4][NT / 32];
     __shared__ long long s_item;
     __shared__ unsigned long long s_passes, s_nc, s_np, s_fb;
-    __shared__ unsigned int s_max;
+    __shared__ unsigned int s_max, s_bad, s_late;
     const Lattice& L = Tr::template lat<N1>();
     const LatticeFix& F = Tr::template lat_fix<N1>();
     const int tid = threadIdx.x;
@@ -394,13 +447,15 @@ __global__ void __launch_bounds__(TXS* TYS* KS, MINB) k_step_fixed(StagedArgs<do
         const int tiles_x = (G.iw + LTX - 1) / LTX;
         const int ltx0 = G.ix0 + (int)(t % tiles_x) * LTX;
         const int lty0 = G.iy0 + (int)(t / tiles_x) * LTY;
-        const int tx0 = ltx0 + sub % SUBX * TXS, ty0 = lty0 + sub / SUBX * TYS;
-        if (SUB > 1 && (tx0 >= G.ix0 + G.iw || ty0 >= G.iy0 + G.ih)) {  // nothing of a ragged tile
+        const int tx0 = ltx0 + sub * TXS, ty0 = lty0;
+        if (SUB > 1 && tx0 >= G.ix0 + G.iw) {  // nothing of a ragged tile
             if (!A.work_counter) break;
             continue;
         }
+        if (tid == 0) s_bad = s_late = 0u;
         const int X = tx0 + n % TXS, Y = ty0 + n / TXS;
-        const bool valid = X < G.ix0 + G.iw && Y < G.iy0 + G.ih;
+        const unsigned group = 1u << (n % TXS / 8);
+        bool valid = X < G.ix0 + G.iw && Y < G.iy0 + G.ih;
         const long long base = G.offset;
         const long long node = base + (long long)Y * G.nx + X;
         const long long rnode = base + (long long)min(lty0 + LTY / 2, G.iy0 + G.ih - 1) * G.nx +
@@ -446,36 +501,60 @@ __global__ void __launch_bounds__(TXS* TYS* KS, MINB) k_step_fixed(StagedArgs<do
                                   fmaxf(fabsf((float)(rux - pg.ux)), fabsf((float)(ruy - pg.uy))));
             in_range = in_range && de <= kFixTileDe * (float)pg.st;
         }
-        staged_block_minmax4<Tr, NT>(vxlo, vxhi, vylo, vyhi, s_red);
-
-        // staged window in unwrapped grid coordinates (departure = x - v dt)
-        const float m = A.margin;
         const float fdt = (float)A.P.dt;
-        const float bxl = fminf(fmaxf(vxlo, -1.0e6f), 1.0e6f), bxh = fminf(fmaxf(vxhi, -1.0e6f), 1.0e6f);
-        const float byl = fminf(fmaxf(vylo, -1.0e6f), 1.0e6f), byh = fminf(fmaxf(vyhi, -1.0e6f), 1.0e6f);
-        const int wx0 = (int)floorf((float)tx0 - bxh * fdt - m) - 1;
-        const int wx1 = (int)floorf((float)(tx0 + TXS - 1) - bxl * fdt + m) + 2;
-        const int wy0 = (int)floorf((float)ty0 - byh * fdt - m) - 1;
-        const int wy1 = (int)floorf((float)(ty0 + TYS - 1) - byl * fdt + m) + 2;
-        const bool fin = isfinite(vxlo) && isfinite(vxhi) && isfinite(vylo) && isfinite(vyhi) &&
-                         vxlo > -1.0e6f && vxhi < 1.0e6f && vylo > -1.0e6f && vyhi < 1.0e6f;
-        const int ww = fin ? max(1, min(wx1 - wx0 + 1, A.ww)) : 1;
-        const int wh = fin ? max(1, min(min(wy1 - wy0 + 1, A.wh), WN / ww)) : 1;
-        // (displacements in the fixed-point range of fix_departure)
-        in_range = in_range && fin &&
-                   fmaxf(fmaxf(fabsf(vxlo), fabsf(vxhi)), fmaxf(fabsf(vylo), fabsf(vyhi))) * fdt < 400.0f;
+        // (finite, and displacements in the fixed-point range of fix_departure)
+        in_range = in_range && (!valid || (vxlo * fdt > -400.0f && vxhi * fdt < 400.0f &&
+                                           vylo * fdt > -400.0f && vyhi * fdt < 400.0f));
+        staged_block_minmax4<Tr, NT>(vxlo, vxhi, vylo, vyhi, s_red);
+        unsigned bad = 0u;  // groups out of range (uniform)
+        if (__syncthreads_or(!in_range)) {
+            if (!in_range) atomicOr(&s_bad, group);
+            __syncthreads();
+            bad = s_bad;
+            if (NG > 1) {  // the window of the others
+                valid = valid && !(bad & group);
+                const float sp = (float)(A.c_max * pg.st);
+                vxlo = valid ? (float)pg.ux - sp : 3.0e38f;
+                vxhi = valid ? (float)pg.ux + sp : -3.0e38f;
+                vylo = valid ? (float)pg.uy - sp : 3.0e38f;
+                vyhi = valid ? (float)pg.uy + sp : -3.0e38f;
+                staged_block_minmax4<Tr, NT>(vxlo, vxhi, vylo, vyhi, s_red);
+            }
+        }
+        constexpr unsigned ALL = (1u << NG) - 1u;
 
-        // a tile out of range by its gauges is not staged
-        if (!__syncthreads_or(!in_range))
-            in_range = stage_window_fixed<N1, KS == 1>(A.in, A.plane, G, base, wx0, wy0, ww, wh, WN, rux,
-                                                       ruy, rst, kFix - rexp, s_h, s_l, F, c_max,
-                                                       A.stats, tid, NT);
-        else
-            in_range = false;
-        if (__syncthreads_or(!in_range)) {  // also: the window is staged
-            if (tid == 0) A.redo_list[atomicAdd(A.redo_count, 1u)] = (unsigned)item;
-            if (!A.work_counter) break;
-            continue;
+        // staged window in unwrapped grid coordinates (departure = x - v dt); with
+        // no node left in range it is empty and not staged
+        const float m = A.margin;
+        const bool any = vxlo <= vxhi;
+        const int wx0 = any ? (int)floorf((float)tx0 - vxhi * fdt - m) - 1 : 0;
+        const int wx1 = any ? (int)floorf((float)(tx0 + TXS - 1) - vxlo * fdt + m) + 2 : 0;
+        const int wy0 = any ? (int)floorf((float)ty0 - vyhi * fdt - m) - 1 : 0;
+        const int wy1 = any ? (int)floorf((float)(ty0 + TYS - 1) - vylo * fdt + m) + 2 : 0;
+        const int ww = max(1, min(wx1 - wx0 + 1, A.ww));
+        const int wh = max(1, min(min(wy1 - wy0 + 1, A.wh), WN / ww));
+        if (bad != ALL) {
+            const bool ok = stage_window_fixed<N1, KS == 1>(A.in, A.plane, G, base, wx0, wy0, ww, wh, WN,
+                                                            rux, ruy, rst, kFix - rexp, s_h, s_l, F,
+                                                            c_max, A.stats, tid, NT);
+            if (__syncthreads_or(!ok)) {  // also: the window is staged
+                if (NG > 1) {
+                    bad |= fixed_bad_groups<TXS, TYS, NT>(s_h, wx0, wy0, ww, wh, tx0, ty0, m, fdt, valid,
+                                                          (float)pg.ux, (float)pg.uy,
+                                                          (float)(A.c_max * pg.st), n, &s_bad);
+                    valid = valid && !(bad & group);
+                } else {
+                    bad = ALL;
+                }
+            }
+        }
+        if (bad) {
+            if (tid < NG && (bad >> tid & 1u) && tx0 + 8 * tid < G.ix0 + G.iw)
+                A.redo_list[atomicAdd(A.redo_count, 1u)] = (unsigned)(item * NG + tid);
+            if (bad == ALL) {
+                if (!A.work_counter) break;
+                continue;
+            }
         }
 
         // ---------------------------------------------------- pass loop
@@ -490,14 +569,26 @@ __global__ void __launch_bounds__(TXS* TYS* KS, MINB) k_step_fixed(StagedArgs<do
         unsigned int offwin = 0u, off_last = 0u;  // populations of a pass read from global memory
         bool done = !valid;
         while (__any_sync(FULL, !done)) {
-            const bool work = !done;
             const double st = pg.st, ux = pg.ux, uy = pg.uy;
             // target gauge of this pass: its offsets from lambda_r
             const double inv = kFixOne / st;
             const long long rt = __double2ll_rn((rst - st) * inv);
             const long long dxt = __double2ll_rn((rux - ux) * inv);
             const long long dyt = __double2ll_rn((ruy - uy) * inv);
-            const bool near_r = fix_offset(rt, dxt, dyt, c_max) <= kFixNodeDe;
+            if (!done && !(fix_offset(rt, dxt, dyt, c_max) <= kFixNodeDe)) {
+                // the node left the range on the way: to the FP64 form, by its
+                // mark (staged_fallback took it at first, 16 populations one
+                // after the other: 15 such nodes held a step for 4 ms)
+                done = true;
+                valid = false;
+                if (part == 0) {
+                    A.out.st[node] = __longlong_as_double(kRedoMark);
+                    if (!(atomicOr(&s_late, group) & group))
+                        A.redo_list[atomicAdd(A.redo_count, 1u)] =
+                            kRedoMarked | (unsigned)(item * NG + n % TXS / 8);
+                }
+            }
+            const bool work = !done;
             const Fix Rt = fix_split(rt);
             __syncwarp();  // the tables are written again
             if (work) {
@@ -518,7 +609,7 @@ __global__ void __launch_bounds__(TXS* TYS* KS, MINB) k_step_fixed(StagedArgs<do
                     int top = Y - wy0 - 1 + fix_departure(__double2ll_rn(d), ly);
 #pragma unroll
                     for (int j = 0; j < 4; ++j) s_ly[(4 * l + j) * NN + n] = make_int2(ly[j].h, ly[j].l);
-                    if (!(near_r && fabs(d) < 500.0 * kFixDisplacement && top >= 0 && top + 3 < wh))
+                    if (!(fabs(d) < 500.0 * kFixDisplacement && top >= 0 && top + 3 < wh))
                         top = -1;
                     s_top[l * NN + n] = top;
                 }

@@ -191,7 +191,6 @@ struct TileWindow {
     // only bound a tile's choice (0: ww * wh, fww * fwh)
     int wn, fwn;
 };
-inline int window_nodes(const TileWindow& w) { return w.wn ? w.wn : w.ww * w.wh; }
 
 // Mixed-precision step over one or many grids (one CTA per tile; batched
 // contexts use a persistent work list).
@@ -206,7 +205,7 @@ cudaError_t launch_step_mixed(const StateBuf<float>& in, const StateBuf<float>& 
 // forms, over one or many grids (tiles 32 x ty; ty 4 or 8 in FP64, 4, 8 or
 // 16 in the mixed form), its per-device set-up (returns resident CTAs per SM
 // for a dynamic shared-memory size) and that size for a window.
-// redo: the FP64 form's {count, exit count, tile list} of n_tiles + 2 words,
+// redo: the FP64 form's {count, exit count, list} of 4 n_tiles + 2 words,
 // the first two zero before the first launch (each launch leaves them zero).
 cudaError_t launch_step_staged_fp64(const StateBuf<double>& in, const StateBuf<double>& out,
                                     int32_t* iters, DevStats* stats, const GridDesc* grids_dev,
@@ -242,7 +241,7 @@ inline int window_extent(double span, double dt, double pad) {
 // (as staged_smem_bytes: the FP64 form also holds the y-map table)
 inline size_t staged_window_bytes(const TileWindow& w) {
     const size_t per_node = w.real_bytes == 8 ? 2 : 1;
-    return (size_t)w.n1 * window_nodes(w) * 4 * w.real_bytes +
+    return (size_t)w.n1 * w.ww * w.wh * 4 * w.real_bytes +
            per_node * w.n1 * w.n1 * w.tx * w.ty * w.real_bytes;
 }
 constexpr int STAGED_TY_FP64[2] = {4, 8};

@@ -64,6 +64,11 @@ struct __align__(32) Double4 {
     double x, y, z, w;
 };
 
+// A part on the redo list with this bit: only its nodes whose output gauge
+// k_step_fixed marked (bits of a NaN that no arithmetic makes).
+constexpr unsigned kRedoMarked = 0x80000000u;
+constexpr long long kRedoMark = 0x7ff4706f6e645f31ll;
+
 template <typename Real>
 struct StagedArgs {
     StateBuf<Real> in, out;
@@ -76,11 +81,10 @@ struct StagedArgs {
     long long n_tiles;
     long long plane;  // plane stride of the packed state
     unsigned int* work_counter;
-    // tiles k_step_fixed left to k_step_staged<StagedFP64>: {count, CTAs of the
-    // redo launch that have exited}, and the tiles (FP64 form only)
+    // what k_step_fixed left to k_step_staged<StagedFP64>: {count, CTAs of the
+    // redo launch that have exited}, and the parts of 8 columns (FP64 form only)
     unsigned int* redo_count;
-    unsigned int* redo_list;  // entries tile * (sub_x * sub_y) + sub
-    int sub_x, sub_y;         // parts of a tile that k_step_fixed's CTAs take
+    unsigned int* redo_list;  // entries 4 * tile + column / 8 (+ kRedoMarked)
     int ww, wh, wn;   // largest window a tile may stage: sides, nodes (FP64 form)
     double c_max;
     float margin;
@@ -259,12 +263,16 @@ __device__ __forceinline__ void stage_window(const StateBuf<typename Tr::Real>& 
     }
 }
 
-// KS = 1: a thread per node of the TX x TY tile.  KS = 2 or 4 (mixed form, small
-// grids): a CTA takes a part of TXS = 32 / KS columns with KS lanes per node, lane
-// `part` sweeping the x-speeds k = part, part + KS, ..; 32 / KS >= 8 nodes stand
-// side by side, so the 16-byte reads of a quarter warp stay contiguous.  The same
-// sums in the same order (over l per x-speed, then over the x-speeds): a grid's
-// result does not depend on KS.
+// KS = 1: a thread per node of the TX x TY tile.  KS = 2 or 4: a CTA takes a part
+// of TXS = 32 / KS columns with KS lanes per node, lane `part` sweeping the
+// x-speeds k = part, part + KS, ..; 32 / KS >= 8 nodes stand side by side, so the
+// 16-byte reads of a quarter warp stay contiguous.  The same sums in the same
+// order (over l per x-speed, then over the x-speeds): a grid's result does not
+// depend on KS.  The mixed form takes lanes for small grids.  The FP64 form runs
+// only what k_step_fixed left, parts of 8 columns with four lanes: the chain of
+// passes is what such a launch waits for (44x66 vortex, the launch over the
+// left-over parts: 2.0 ms as rows of a 32-wide tile, about 2 ms with a thread per
+// node in two warps, 0.62 ms with four lanes; the whole step in FP64: 1.9 ms).
 template <class Tr, int TX, int TY, int N1, int KS = 1, int TXS = TX>
 __global__ void __launch_bounds__(TXS* TY* KS, Tr::template min_blocks<TXS * TY * KS>())
 k_step_staged(StagedArgs<typename Tr::Real> A) {
@@ -272,13 +280,13 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
     using Real4 = typename Tr::Real4;
     constexpr int NN = TXS * TY, NT = NN * KS, SUB = TX / TXS;
     constexpr unsigned FULL = 0xffffffffu;
-    static_assert(TX == 32 && (KS == 1 ? TXS == 32 : Tr::kPacked && TXS * KS == 32 && !Tr::kEyTable),
-                  "a warp is one tile row, or quarter warps are");
+    static_assert(TX == 32 && TXS * KS == 32 && (!Tr::kRedo || KS == 4),
+                  "a warp is one tile row or rows of parts");
     extern __shared__ __align__(32) unsigned char smem_raw[];
     const int WN = Tr::kRedo ? A.wn : A.ww * A.wh;
     Real4* s_f = reinterpret_cast<Real4*>(smem_raw);              // [N1][WN]: row a of g
     Real* s_acc = reinterpret_cast<Real*>(s_f + (size_t)N1 * WN);  // [Q][NN]
-    Real* s_ey = s_acc + (size_t)N1 * N1 * NN;  // [Q][NT] Ey[l][b] of the pass (kEyTable)
+    Real* s_ey = s_acc + (size_t)N1 * N1 * NN;  // [Q][NN] Ey[l][b] of the pass (kEyTable)
     __shared__ float s_red[4][NT / 32];
     __shared__ long long s_item;
     __shared__ unsigned long long s_passes, s_nc, s_np, s_fb;
@@ -299,18 +307,18 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
     const unsigned long long t_begin = (A.work_counter && tid == 0) ? pond_globaltimer() : 0ull;
 
     long long item = blockIdx.x;
-    // the redo launch takes its tiles from the list k_step_fixed left
-    const bool redo = Tr::kRedo && A.redo_count != nullptr;
+    // the redo launch takes its parts from the list k_step_fixed left
+    constexpr bool redo = Tr::kRedo;
     unsigned int redo_i = blockIdx.x;
-    int redo_sub = 0;
+    bool marked = false;
     const unsigned int redo_n = redo ? *A.redo_count : 0u;
     for (;;) {
-        if (redo) {
+        if constexpr (redo) {
             if (redo_i >= redo_n) break;
-            item = A.redo_list[redo_i];
+            const unsigned e = A.redo_list[redo_i];
+            item = e & ~kRedoMarked;
+            marked = (e & kRedoMarked) != 0u;
             redo_i += gridDim.x;
-            redo_sub = (int)(item % (A.sub_x * A.sub_y));
-            item /= A.sub_x * A.sub_y;
         } else if (A.work_counter) {
             __syncthreads();
             if (tid == 0) s_item = (long long)atomicAdd(A.work_counter, 1u);
@@ -338,16 +346,15 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
         const int ltx0 = G.ix0 + (int)(t % tiles_x) * TX, tx0 = ltx0 + sub * TXS;
         const int ty0 = G.iy0 + (int)(t / tiles_x) * TY;
         if (SUB > 1 && tx0 >= G.ix0 + G.iw) {  // nothing of a ragged tile
-            if (!A.work_counter) break;
+            if (!redo && !A.work_counter) break;
             continue;
         }
         const int X = tx0 + lxi, Y = ty0 + lyi;
         bool valid = X < G.ix0 + G.iw && Y < G.iy0 + G.ih;
-        if (redo)  // only the part of the tile that was left over
-            valid = valid && lxi / (TX / A.sub_x) == redo_sub % A.sub_x &&
-                    lyi / (TY / A.sub_y) == redo_sub / A.sub_x;
         const long long base = G.offset;
         const long long node = base + (long long)Y * G.nx + X;
+        if constexpr (redo)
+            valid = valid && !(marked && __double_as_longlong(A.out.st[node]) != kRedoMark);
 
         // reference gauge lambda_r of the tile: its centre node (clamped to
         // the interior), so the staged sources' gauges differ from lambda_r by
@@ -423,16 +430,18 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
             if constexpr (Tr::kEyTable) {
                 // the y-map r -> lambda of this pass, Ey[l][b] in correction
                 // form, for every x-speed
+                __syncwarp();  // the lanes of a node are done with the last pass's
                 if (work) {
-#pragma unroll
-                    for (int l = 0; l < N1; ++l)
+#pragma unroll 1
+                    for (int l = part; l < N1; l += KS)
 #pragma unroll
                         for (int b = 0; b < N1; ++b) {
                             const Real de = fma((Real)L.c[b], rt, dyt);
-                            s_ey[(N1 * l + b) * NT + tid] =
+                            s_ey[(N1 * l + b) * NN + n] =
                                 gauge_tail<N1>((Real)L.d3[l], (Real)L.d2[l][b], (Real)L.d1[l][b], de) * de;
                         }
                 }
+                __syncwarp();
             }
             // y-stencils of the n1 y-speeds: top row in the window and weights
             int top[N1];
@@ -650,7 +659,7 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
                             for (int b = 0; b < N1; ++b) {
                                 Real ey;
                                 if constexpr (Tr::kEyTable) {
-                                    ey = s_ey[(N1 * l + b) * NT + tid];
+                                    ey = s_ey[(N1 * l + b) * NN + n];
                                 } else {
                                     const Real de = fma((Real)L.c[b], rt, dyt);
                                     ey = gauge_tail<N1>((Real)L.d3[l], (Real)L.d2[l][b],
@@ -721,7 +730,7 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
             atomicAdd(&s_passes, (unsigned long long)wsum);
             atomicMax(&s_max, wmax);
         }
-        if (!A.work_counter && !redo) break;
+        if (!redo && !A.work_counter) break;
         __syncthreads();  // the next item restages the window
     }
     __syncthreads();

@@ -1,3 +1,4 @@
+#include <algorithm>
 // pond_step_fp64.cu -- FP64 PonD time step of one periodic grid.
 //
 // This file holds the direct FP64 kernels (described here; contexts with
@@ -581,7 +582,7 @@ struct StagedFP64 {
     static constexpr bool kEyTable = true;
     template <int NT>
     static constexpr int min_blocks() {
-        return NT >= 256 ? 1 : 2;
+        return 256 / NT;
     }
     template <int N1>
     static __device__ __forceinline__ const Lattice& lat() {
@@ -736,10 +737,13 @@ static const FixedShape kFixedShapes[] = {
 };
 constexpr int kFixedShapeCount = sizeof(kFixedShapes) / sizeof(kFixedShapes[0]);
 
-static void (*staged64_kernel(int ty, int n1))(StagedArgs<double>) {
-    if (n1 == 3) return ty == 4 ? k_step_staged<StagedFP64, 32, 4, 3> : k_step_staged<StagedFP64, 32, 8, 3>;
-    return ty == 4 ? k_step_staged<StagedFP64, 32, 4, 4> : k_step_staged<StagedFP64, 32, 8, 4>;
+// The FP64 kernel of the parts of 8 columns that the fixed-point one leaves.
+static void (*left_kernel(int ty, int n1))(StagedArgs<double>) {
+    if (n1 == 3)
+        return ty == 4 ? k_step_staged<StagedFP64, 32, 4, 3, 4, 8> : k_step_staged<StagedFP64, 32, 8, 3, 4, 8>;
+    return ty == 4 ? k_step_staged<StagedFP64, 32, 4, 4, 4, 8> : k_step_staged<StagedFP64, 32, 8, 4, 4, 8>;
 }
+static size_t left_bytes(const TileWindow& w) { return staged_smem_bytes(w.n1, w.wn, 1, 8 * w.ty, 8); }
 
 static size_t fixed_bytes(const TileWindow& w) {
     return fixed_smem_bytes(w.n1, w.fwn ? w.fwn : w.fww * w.fwh, w.fx * w.fy);
@@ -770,6 +774,11 @@ static int fixed_widest(int n1, int ty, int64_t n_tiles, int sms) {
 
 constexpr size_t kFixedSmemCap = 225 * 1024, kStagedSmemCap = 220 * 1024;
 
+// nodes of the window that a left-over part can stage in `bytes`
+static int left_capacity(int n1, int ty, size_t bytes) {
+    return (int)((bytes - staged_smem_bytes(n1, 0, 1, 8 * ty, 8)) / ((size_t)n1 * 32));
+}
+
 // Per-device set-up of the window's two kernels: the resident CTAs per SM of
 // the fixed-point one.
 static cudaError_t fixed_attributes(const TileWindow& win, int pick, int* ctas_per_sm) {
@@ -778,7 +787,7 @@ static cudaError_t fixed_attributes(const TileWindow& win, int pick, int* ctas_p
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    e = raise_smem(staged64_kernel(win.ty, win.n1), staged_window_bytes(win),
+    e = raise_smem(left_kernel(win.ty, win.n1), left_bytes(win),
                    &s_left[dev][(win.n1 == 3 ? 2 : 0) + (win.ty == 8 ? 1 : 0)]);
     if (e != cudaSuccess) return e;
     const FixedShape& f = kFixedShapes[pick];
@@ -809,6 +818,7 @@ cudaError_t staged_prepare_fp64(TileWindow* win, int ex, int ey, int64_t n_tiles
     while (fixed_bytes(*win) > kFixedSmemCap) {
         if (win->fww - win->fx >= win->fwh - win->fy) --win->fww; else --win->fwh;
     }
+    win->wn = std::min((8 + ex) * (ty + ey), left_capacity(n1, ty, kStagedSmemCap));
     return fixed_attributes(*win, pick, ctas_per_sm);
 }
 
@@ -816,8 +826,6 @@ cudaError_t staged_prepare_fp64(TileWindow* win, int ex, int ey, int64_t n_tiles
 // none; its CTAs then end at once).
 static cudaError_t launch_fixed(StagedArgs<double> A, const TileWindow& win, int persistent_ctas,
                                 cudaStream_t s) {
-    A.sub_x = win.tx / win.fx;
-    A.sub_y = win.ty / win.fy;
     A.ww = win.fww;
     A.wh = win.fwh;
     A.wn = win.fwn ? win.fwn : win.fww * win.fwh;
@@ -825,7 +833,7 @@ static cudaError_t launch_fixed(StagedArgs<double> A, const TileWindow& win, int
     for (const FixedShape& c : kFixedShapes)
         if (c.n1 == win.n1 && c.ty == win.ty && c.fx == win.fx && c.fy == win.fy && c.ks == win.fks) f = &c;
     if (!f) return cudaErrorInvalidValue;
-    const int64_t parts = A.n_tiles * A.sub_x * A.sub_y;
+    const int64_t parts = A.n_tiles * (win.tx / win.fx);
     unsigned int nb = parts > 0 ? (unsigned int)parts : 1u;
     if (A.work_counter) {
         cudaError_t e = cudaMemsetAsync(A.work_counter, 0, sizeof(unsigned int), s);
@@ -835,12 +843,11 @@ static cudaError_t launch_fixed(StagedArgs<double> A, const TileWindow& win, int
     f->kern<<<nb, f->fx * f->fy * f->ks, fixed_bytes(win), s>>>(A);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    A.ww = win.ww;
-    A.wh = win.wh;
-    A.wn = window_nodes(win);
-    nb = (unsigned int)(persistent_ctas < A.n_tiles ? persistent_ctas : A.n_tiles);
-    if (nb < 1u) nb = 1u;
-    staged64_kernel(win.ty, win.n1)<<<nb, 32 * win.ty, staged_window_bytes(win), s>>>(A);
+    A.ww = A.wh = win.wn;  // by the nodes
+    A.wn = win.wn;
+    const int64_t left = std::min<int64_t>(4 * A.n_tiles, persistent_ctas);
+    nb = left > 0 ? (unsigned int)left : 1u;
+    left_kernel(win.ty, win.n1)<<<nb, 32 * win.ty, left_bytes(win), s>>>(A);
     return cudaGetLastError();
 }
 
@@ -971,8 +978,7 @@ static TileWindow noalloc_window(int n1, int64_t n_tiles_8, int64_t n_tiles_4, i
     // two CTAs per SM for the shapes of two
     const size_t cap = w.fx * w.fy * w.fks < 256 ? kFixedSmemCap / 2 : kFixedSmemCap;
     w.fwn = (int)((cap - fixed_smem_bytes(n1, 0, w.fx * w.fy)) / ((size_t)n1 * 32));
-    const size_t tables = 2 * sizeof(double) * n1 * n1 * w.tx * w.ty;
-    w.wn = (int)((kStagedSmemCap - tables) / ((size_t)n1 * 32));
+    w.wn = left_capacity(n1, w.ty, kStagedSmemCap);
     w.ww = w.fww = 256;
     w.wh = w.fwh = 256;
     return w;
@@ -1081,7 +1087,7 @@ extern "C" pond_status pond_step_fp64_noalloc(const pond_config* cfg, int32_t nx
         // the staged step, as a context runs it by default (200 x 150: 4.86 ms
         // with one node per thread of the direct kernel, 0.34 ms so); its list of left-over
         // tiles goes into T_out, which nothing else touches before the end
-        // (a tile has at least one node, so the list fits)
+        // (a part has at least one node, so the list fits)
         StagedArgs<double> A{};
         A.in = in;
         A.out = out;

@@ -49,6 +49,12 @@ def field(name, nx, ny, T_L):
         f.rho = np.exp(3.0 * np.sin(2 * np.pi * x)) * np.ones((ny, 1))
     if name == "shear":    # gauge spreads on both sides of the tile limit
         f.ux = f.ux + 0.5 * np.sin(2 * np.pi * y) ** 3 * np.ones((1, nx))
+    if name == "spots":    # parts of tiles out of range by gauge, and by a dense source
+        x, y = np.arange(nx)[None, :], np.arange(ny)[:, None]
+        f.ux = f.ux + 0.7 * np.exp(-((x - nx // 3) ** 2 + (y - ny // 2) ** 2) / 8.0)
+        f.rho = f.rho * (1.0 + 60.0 * np.exp(-((x - nx // 2) ** 2 + (y - ny // 3) ** 2) / 8.0))
+    if name == "vortex":   # nodes that leave the range in a pass
+        f = workloads.vortex(nx, 0.1 * nx, 0.5, 1.0)
     c = np.sqrt(T_L)
     return workloads.Fields(f.rho, f.ux * c, f.uy * c, f.T * T_L)
 
@@ -56,7 +62,8 @@ def field(name, nx, ny, T_L):
 @pytest.mark.parametrize("lattice", [pond.POND_D2Q16, pond.POND_D2Q9])
 @pytest.mark.parametrize("tile_rows", [4, 8])
 @pytest.mark.parametrize("name,nx,ny", [("plain", 31, 7), ("plain", 33, 9), ("plain", 64, 17),
-                                        ("density", 160, 12), ("shear", 40, 64)])
+                                        ("density", 160, 12), ("shear", 40, 64),
+                                        ("spots", 100, 30), ("vortex", 44, 44)])
 def test_matches_oracle(name, nx, ny, tile_rows, lattice):
     T_L = 1.0 / 3.0 if lattice == pond.POND_D2Q9 else 1.0
     against_oracle(field(name, nx, ny, T_L), 2, lattice, tile_rows=tile_rows)
@@ -79,9 +86,10 @@ def test_scaled_populations_scale_the_result_exactly(power):
     (pond.POND_D2Q16, 8, 256, 176, 1, 2),   # 176 half tiles against 88 by parts
     (pond.POND_D2Q16, 4, 256, 128, 2, 2),   # 256 against 64, four rows
     (pond.POND_D2Q9, 8, 512, 160, 2, 2), (pond.POND_D2Q9, 4, 256, 128, 2, 2)])
-def test_parts_of_tiles_match_whole_tiles_bit_for_bit(lattice, tile_rows, nx, ny, px, py):
+@pytest.mark.parametrize("name", ["plain", "spots"])
+def test_parts_of_tiles_match_whole_tiles_bit_for_bit(name, lattice, tile_rows, nx, ny, px, py):
     T_L = 1.0 / 3.0 if lattice == pond.POND_D2Q9 else 1.0
-    fields = field("plain", nx, ny, T_L)
+    fields = field(name, nx, ny, T_L)
     cfg = dict(lattice=lattice, T_ref=T_L)
     whole, _ = run(fields, 2, tile_rows=tile_rows, **cfg)
     with decomp.DecomposedSim(nx, ny, px, py, 14, precision=pond.POND_FP64, tile_rows=tile_rows,
