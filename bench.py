@@ -80,19 +80,31 @@ def staged_flops_per_pass(n1: int, st_mean: float, every_row: bool = False) -> f
     return n1 * per_k + 20 * n1 + 40 + ymap_pass
 
 
+# 64-bit-sum integer multiply-adds (mad.wide.s32) per node-pass of the FP64
+# form, whose contractions run in fixed point on the integer multiplier: three
+# per product.  Per row, the products of the FP64 form above (4 n1^2); per
+# population, its four rows (4 n1) and the y-map (n1).  The maps' entries,
+# the weights and the once-per-step staging are left out: a lower bound.
+def fixed_mads_per_pass(n1: int, st_mean: float) -> float:
+    spread = 2 * 2.3344142183389773 if n1 == 4 else 2.0
+    rows = 4.0 + spread * st_mean
+    return 3 * n1 * (4 * n1 * n1 * rows + n1 * 5 * n1)
+
+
+# Nominal rate of those at the maximum SM clock: 32 a clock and SM (a probe of
+# independent chains measures that rate too), in units of 10^12.
+PEAK_WIDE_MAD = 152 * 32 * 2.07e9 / 1e12
+
 # Nominal peaks of the arithmetic pipes at the 2070 MHz maximum SM clock
 # (FP64 1.25 TFLOP/s; FP32 152 SMs x 128 lanes x 2 flops x 2.07 GHz).  The
 # roofline uses the rates the FMA-chain probe (pond_measure_peak) measures
 # at the start of every run instead; these are the fallback if it fails.
 PEAK_FP64_TFLOPS = 1.25
 PEAK_FP32_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
-# DRAM bytes per FP64 step launch at 2048^2 of the staged kernel: the ncu
-# capture of the same kernel (k_step_staged<StagedFP64, 32, 8, 4>) at 1024^2
-# read 161.5 MB and wrote 125.6 MB; traffic grows with the node count (4x).
-K_STAGED64_TRAFFIC_2048 = 4 * (161.49e6 + 125.57e6)
+# DRAM bytes per FP64 step launch at 2048^2 (an ncu capture of k_step_fixed).
+K_STAGED64_TRAFFIC_2048 = 642.70e6 + 622.76e6
 K_STAGED64_TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one "
-                             "k_step_staged<StagedFP64, 32, 8, 4> launch at 1024^2 (287.1 MB), "
-                             "scaled x4 by nodes to the 2048^2 launch")
+                             "k_step_fixed<StagedFP64, 32, 8, 32, 8, 1, 4> launch at 2048^2")
 
 
 def parse():
@@ -388,6 +400,7 @@ def run_pond(args, world, rank, local):
     sim.step(args.warmup)
     st_mean = float(np.sqrt(fields.T).mean())
     flop_pass = staged_flops_per_pass(4, st_mean)
+    mad_pass = fixed_mads_per_pass(4, st_mean)
     barrier(world)
     with ClockSampler(local) as clk:
         secs, stats = time_steps(sim, stream, args.steps)
@@ -397,7 +410,8 @@ def run_pond(args, world, rank, local):
     rho64, ux64, uy64, T64 = sim.moments()
     mean_passes = stats["passes"] / stats["node_updates"]
     kernel_s = secs / args.steps
-    achieved = flop_pass * (stats["passes"] / args.steps) / kernel_s / 1e12
+    achieved = mad_pass * (stats["passes"] / args.steps) / kernel_s / 1e12
+    flops64 = flop_pass * (stats["passes"] / args.steps) / kernel_s / 1e12
     line = {
         "metric": METRIC,
         "value": world * nodes * args.steps / secs_max,
@@ -418,20 +432,24 @@ def run_pond(args, world, rank, local):
         "mean_passes": mean_passes,
         "max_passes": stats["max_passes"],
         "nonconverged": stats["nonconverged"],
-        "gpu_launches": args.steps,
-        "roofline": {"bound": "alu", "pipe": "fp64", "achieved": achieved,
-                     "peak": peak64, "unit": "TFLOP/s",
-                     "frac": achieved / peak64,
+        "gpu_launches": 2 * args.steps,  # the fixed-point launch and the one over left-over parts
+        "roofline": {"bound": "alu", "pipe": "integer multiply (mad.wide.s32)",
+                     "achieved": achieved,
+                     "peak": PEAK_WIDE_MAD, "unit": "Tmad/s",
+                     "frac": achieved / PEAK_WIDE_MAD,
+                     "mad_per_pass": mad_pass,
+                     "fp64_equivalent_tflops": flops64,
+                     "fp64_equivalent_of_fp64_peak": flops64 / peak64,
                      "traffic": K_STAGED64_TRAFFIC_2048,
                      "traffic_source": K_STAGED64_TRAFFIC_SOURCE,
-                     "peak_source": peak_src,
-                     "peak_nominal": PEAK_FP64_TFLOPS,
-                     "flop_per_pass": flop_pass,
-                     "flop_count": "staged kernel, per-pass sweep only (staging excluded)",
+                     "peak_source": "nominal: 32 per clock and SM at 2070 MHz",
+                     "fp64_peak": peak64, "fp64_peak_source": peak_src,
+                     "fp64_flop_per_pass": flop_pass,
+                     "count": "staged kernel, per-pass sweep only (staging excluded)",
                      "direct_equivalent_tflops": FLOP_PER_PASS * (stats["passes"] / args.steps)
                                                  / kernel_s / 1e12,
                      "tile": [32, stats.get("tile_rows", 0)],
-                     "kernel": "k_step_staged<StagedFP64>", "kernel_ms": kernel_s * 1e3,
+                     "kernel": "k_step_fixed<StagedFP64>", "kernel_ms": kernel_s * 1e3,
                      "hbm_gbs_algorithmic": nodes * BYTES_FP64 / kernel_s / 1e9,
                      "hbm_peak_gbs": peaks.get("hbm_gbs")},
         "clocks": clocks,
@@ -561,6 +579,11 @@ def run_pond(args, world, rank, local):
                                    staged_flops_per_pass(3, float(np.sqrt(q9.T * 3.0).mean()),
                                                          every_row=prec != pond.POND_FP64),
                                    FLOP_PER_PASS_Q9)
+            if prec == pond.POND_FP64:  # contractions on the integer multiplier
+                mads = fixed_mads_per_pass(3, float(np.sqrt(q9.T * 3.0).mean()))
+                forms[key].update(fp64_equivalent_of_fp64_peak=forms[key].pop("alu_frac"),
+                                  mad_per_pass=mads,
+                                  alu_frac=mads * qstats["passes"] / qsecs / 1e12 / PEAK_WIDE_MAD)
             q9_out[key] = qsim.moments()
             qsim.close()
         r64, u64x, u64y, t64 = q9_out["fp64_d2q9_2048"]

@@ -71,7 +71,10 @@ enum { POND_KERNEL_DEFAULT = 0, POND_KERNEL_STAGED = 1, POND_KERNEL_DIRECT = 2 }
 
 /* Run configuration.  Fill with pond_config_default() and override. */
 typedef struct pond_config {
-    int32_t precision;  /* POND_FP64: all arithmetic and storage FP64.
+    int32_t precision;  /* POND_FP64: all storage FP64; arithmetic FP64, the
+                           staged kernel's contractions in 64-bit fixed
+                           point where a tile's magnitudes and gauges allow
+                           (errors no larger than FP64's), else FP64.
                            POND_FP32_MIXED: populations and bulk arithmetic
                            FP32; gauges stored and accumulated in FP64; the
                            gauge differences of the transform formed from the
@@ -137,7 +140,9 @@ typedef struct pond_config {
                            a quarter (mixed) to a fifth (FP64) of the
                            per-pass arithmetic.  Tile
                            shapes 32 x 4 and 32 x 8 nodes (FP64), 32 x 4,
-                           32 x 8, 32 x 16 (mixed).
+                           32 x 8, 32 x 16 (mixed).  Small grids run a tile
+                           by parts with several lanes per node; a grid's
+                           result does not depend on that.
                            POND_KERNEL_DIRECT: the per-(population, source)
                            kernels, G(s -> t) for every stencil node of
                            every population (FP64 mappings by
@@ -179,7 +184,9 @@ void pond_config_default(pond_config* cfg, int32_t precision);
 /* Create a context for n_grids independent periodic grids of sizes
  * nx[g] x ny[g] (n_grids == 1: single grid; > 1: batched ensemble advanced
  * together by one launch per step).  cuda_stream is a cudaStream_t (NULL =
- * legacy default stream).  Allocates the device state; the only later
+ * legacy default stream).  Allocates the device state (and, for the
+ * staged FP64 step, 4 bytes per 8 x 4 nodes for its list of left-over parts);
+ * the only later
  * allocations are a staging area for host buffers (20 FP64 values per node,
  * made by the first call that passes host pointers and grown for a larger
  * grid) and the adjoint's scratch (pond_adjoint_step's first call).
@@ -373,8 +380,9 @@ pond_status pond_step_fp64_noalloc(const pond_config* cfg, int32_t nx, int32_t n
 enum { POND_PIPE_FP64 = 0, POND_PIPE_FP32 = 1, POND_PIPE_FP32X2 = 2 };
 
 /* Measurement utility; the paper has no counterpart.  The PonD step is
- * bound by plain FMA arithmetic (FP64 pipe for the FP64 form, FP32 pipe for
- * the mixed form), so its roofline denominators are FMA rates.  This times
+ * bound by arithmetic (the direct FP64 form by the FP64 pipe, the staged FP64
+ * form by the integer multiplier, the mixed form by FP32 and shared memory);
+ * the FMA rates are the denominators of its rooflines.  This times
  * one launch (after a warm-up launch) of a kernel in which every thread of
  * a grid of (SM count x resident CTAs per SM) CTAs of 256 threads runs eight
  * independent FMA chains for iters x 16 steps, on the current device and

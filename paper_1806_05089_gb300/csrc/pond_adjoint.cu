@@ -22,16 +22,18 @@
 // The seed gauge gets no gradient: the limit does not depend on it.
 //
 // Phase A forms A*, the JVP A_lambda in three directions, the 3 x 3 solve
-// and w.  Contexts on the staged forward kernel run it staged
-// (k_adjoint_jvp_staged: one thread per target node, the sources staged per
-// tile in a reference gauge, then k_adjoint_epilogue); contexts on the
-// direct kernels run k_adjoint_targets (one warp per target node, lane =
-// population).  Phase B (one warp per source node) gathers the transpose
-// over the targets whose departure stencils can contain the source (a
-// window bounded by the particle-velocity range), so the result is
-// deterministic and needs no atomics: per population in the direct
-// contexts (k_adjoint_sources), per target with the target's hit set
-// K x L in the staged ones (k_adjoint_sources_t).
+// and w.  Contexts on the staged forward kernel run it staged, the sources
+// staged per tile in a reference gauge and one thread per target node
+// (k_adjoint_jvp_fixed in fixed point, k_adjoint_jvp_staged in FP64 for the
+// tiles out of its range, then k_adjoint_epilogue); contexts on the direct
+// kernels run k_adjoint_targets (one warp per target node, lane = population).
+// Phase B is the transpose: the staged contexts scatter each target's cotangent
+// over its stencils in fixed point (k_adjoint_scatter, whole-number sums in
+// shared memory, so the order of the additions does not matter and the result
+// is deterministic, then k_adjoint_reduce), and gather over the targets of the
+// tiles out of range (k_adjoint_sources_t: one warp per source node, per target
+// the hit set K x L); the direct contexts gather per population
+// (k_adjoint_sources).
 #include <cmath>
 
 #include "pond_device.cuh"

@@ -1,8 +1,8 @@
 // pond_fixed.cuh -- the FP64 staged step with its contractions in 64-bit
 // fixed point on the integer multiply pipe.
 //
-// GB300 runs 2 FP64 FMAs per clock and SM but 64 integer multiply-adds with a
-// 64-bit sum (mad.wide.s32, measured 60 per clock and SM).  The staged step
+// GB300 runs 2 FP64 FMAs per clock and SM but 32 integer multiply-adds with a
+// 64-bit sum (mad.wide.s32; both measured).  The staged step
 // (pond_staged.cuh) spends four fifths of its FP64 operations on dot products
 // of 16 staged populations with 16 weights; here those run as
 //   sum w g = 2^64 sum w1 g1 + 2^32 sum (w1 g0 + w0 g1) + sum w0 g0,
@@ -17,18 +17,19 @@
 // to R 2^-60 and weights to 2^-60.  A row sum then carries about R 2^-59
 // (2^-54 M or less), where the FP64 sum of 16 products rounds at 2^-53 of its
 // terms: the fixed-point form is the more exact one as long as a tile's
-// populations stay within its window of magnitudes.  So a tile takes this path only if
+// populations stay within its window of magnitudes.  So a group of 8 columns of a tile takes this
+// path only if
 //   - every staged |f| < R / 4 and |g| < R / 4, and at every staged node the
 //     largest |g| is >= R / 128;
 //   - the gauges of its nodes differ from the reference gauge by |xi_a - c_a|
-//     <= 0.52, those of its sources by 1.2 (a pass gauge beyond 0.58 sends that
-//     node to the global-memory path).  With S <= 4.4 the sum of the absolute
+//     <= 0.52, those of its sources by 1.2 (a node whose pass gauge goes beyond
+//     0.58 is marked and computed again).  With S <= 4.4 the sum of the absolute
 //     entries of a map's row at 0.58 and 1.25 that of the cubic weights, every
 //     population stays below 0.4 S^2 R < 8 R and every middle sum below 2^63;
 //   - its displacements are below 400 nodes.
-// Any other tile (strong shear at the window's scale, near-vacuum, NaN, the
+// Any other group (strong shear at the window's scale, near-vacuum, NaN, the
 // seed modes that start far from the reference) is put on a list, and
-// k_step_staged<StagedFP64> runs the listed tiles in a launch that follows.
+// k_step_staged<StagedFP64> runs the listed ones in a launch that follows.
 //
 // The staging, the maps' entries, the cubic weights and the closing re-gauge
 // are in fixed point too: a product of two weights costs about ten
@@ -40,9 +41,9 @@
 // Measured, GB300 (FP64: k_step_staged; contractions: only the dot products in
 // fixed point; all: as here):
 //                                  FP64  contractions      all
-//   2048^2 supersonic, 1 step      69.8          36.8     22.6 ms
-//   301 x 211, 4 steps              7.1           3.6      2.3 ms
-//   1024^2 D2Q9, 2 steps           14.4           8.8      4.9 ms
+//   2048^2 supersonic, 1 step      69.8          36.8     22.1 ms
+//   301 x 211, 4 steps              7.1           3.6      2.2 ms
+//   1024^2 D2Q9, 2 steps           14.4           8.8      4.8 ms
 //   64^2 Taylor-Green, 20 steps    14.0           7.3      1.7 ms
 // It is bound by the integer multiplier: mad.wide runs at 32 a clock and SM
 // (k_step_fixed at 2048^2: 62 % of the time in the row sweep, whose 192 of them

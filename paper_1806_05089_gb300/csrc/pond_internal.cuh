@@ -187,8 +187,8 @@ struct TileWindow {
     // staged window
     int fx, fy, fks;
     int fww, fwh;
-    // nodes of the two windows, when they are set by capacity and the sides
-    // only bound a tile's choice (0: ww * wh, fww * fwh)
+    // FP64 form: nodes of a left-over part's window, and of the fixed-point
+    // kernel's where that is set by capacity (0: fww * fwh)
     int wn, fwn;
 };
 

@@ -1,5 +1,6 @@
-// pond_staged.cuh -- the reference-gauge staged PonD step kernel, for the FP64
-// form (Real = double) and the mixed form (Real = float).
+// pond_staged.cuh -- the reference-gauge staged PonD step kernel: the mixed form
+// (Real = float), and the FP64 form (Real = double) of what pond_fixed.cuh, the
+// FP64 step with its contractions in fixed point, leaves to it.
 //
 // The gauge transform of Eq. transform is a composition: for any reference
 // gauge lambda_r, M_t^-1 M_s = (M_t^-1 M_r)(M_r^-1 M_s), because the Q
@@ -34,11 +35,11 @@
 // form apply them in correction form f + E f, so rounding never touches the
 // identity part; the FP64 form folds Gx(r->t)[k][a] into the x-weights
 // (lx_k[jx] Gx[k][a], once per x-speed and pass), takes the pass's Ey
-// entries from a per-thread shared-memory table, and accumulates each
+// entries from a shared-memory table, and accumulates each
 // population once over its four stencil rows from a four-row buffer of P.
 //
-// One CTA per TX x TY tile (TX = 32: a warp is one tile row of 32 nodes);
-// batched ensembles take (grid, tile) items from an atomic counter.  The pass
+// One CTA per TX x TY tile (TX = 32: a warp is one tile row of 32 nodes), or per
+// part of one with several lanes per node (below); batched ensembles take (grid, tile) items from an atomic counter.  The pass
 // loop is warp-synchronous: the row sweep's bounds are the union over the
 // warp's active lanes (__reduce_min/max_sync), lanes whose node has converged
 // idle, and a lane's populations take only the rows of their own stencils.
@@ -47,7 +48,7 @@
 //
 // Tr (the including translation unit's traits) provides:
 //   Real, Real4 (16 or 32 bytes), kUnrollK, kPacked (the packed FP32 sweep),
-//   kRedo (the kernel runs k_step_fixed's left-over tiles), kEyTable (the Ey
+//   kRedo (the kernel runs k_step_fixed's left-over parts), kEyTable (the Ey
 //   table in shared memory), min_blocks<threads>(), lat<N1>() (lattice
 //   constants of that unit's constant bank), departure (the floor of a
 //   displacement and the cubic weights at its fraction), load4 / store4,

@@ -1,11 +1,10 @@
-#include <algorithm>
 // pond_step_fp64.cu -- FP64 PonD time step of one periodic grid.
 //
 // This file holds the direct FP64 kernels (described here; contexts with
-// kernel = POND_KERNEL_DIRECT, and the allocation-free entry point at the
-// end of the file), the FP64 traits of the reference-gauge staged kernel of
-// pond_staged.cuh (StagedFP64, which FP64 contexts run by default), and that
-// entry point.
+// kernel = POND_KERNEL_DIRECT), the FP64 traits and launches of the
+// reference-gauge staged step (StagedFP64: k_step_fixed of pond_fixed.cuh, then
+// k_step_staged over what that leaves; FP64 contexts run it by default), and the
+// allocation-free entry point, which runs the staged step too.
 //
 // The direct kernels, both bound by the FP64 pipe, all source reads through
 // the read-only L1 path, templated on the lattice (D2Q16, N1 = 4, or D2Q9,
@@ -39,6 +38,7 @@
 // relaxation f + 2 beta (rho W - f) (Eq. postcollision).
 #include <cuda.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "pond_device.cuh"
