@@ -264,12 +264,22 @@ __device__ __forceinline__ void stage_window(const StateBuf<typename Tr::Real>& 
     }
 }
 
+// adds population (k, l) to the sums of f, c_k f, c_l f and |c|^2 f
+template <class Lat, typename Real>
+__device__ __forceinline__ void add_moments(const Lat& L, int k, int l, Real f, Real& m0, Real& m1,
+                                            Real& m2, Real& m3) {
+    const Real ck = (Real)L.c[k], cl = (Real)L.c[l];
+    m0 += f;
+    m1 = fma(ck, f, m1);
+    m2 = fma(cl, f, m2);
+    m3 = fma(fma(ck, ck, cl * cl), f, m3);
+}
+
 // KS = 1: a thread per node of the TX x TY tile.  KS = 2 or 4: a CTA takes a part
 // of TXS = 32 / KS columns with KS lanes per node, lane `part` sweeping the
 // x-speeds k = part, part + KS, ..; 32 / KS >= 8 nodes stand side by side, so the
 // 16-byte reads of a quarter warp stay contiguous.  The same sums in the same
-// order (over l per x-speed, then over the x-speeds): a grid's result does not
-// depend on KS.  The mixed form takes lanes for small grids.  The FP64 form runs
+// order: a grid's result does not depend on KS.  The mixed form takes lanes for small grids.  The FP64 form runs
 // only what k_step_fixed left, parts of 8 columns with four lanes: the chain of
 // passes is what such a launch waits for (44x66 vortex, the launch over the
 // left-over parts: 2.0 ms as rows of a 32-wide tile, about 2 ms with a thread per
@@ -648,8 +658,6 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
                         for (int b = 0; b < N1; ++b) Z[l][b] = z4[b];
                     }
                 }
-                // sums over l of f, c_l f and |c|^2 f, then over the x-speeds in order
-                Real a0 = 0, a2 = 0, a3 = 0;
                 if (work && mine) {
 #pragma unroll
                     for (int l = 0; l < N1; ++l) {
@@ -672,26 +680,23 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
                             offwin |= 1u << (N1 * k + l);
                         }
                         s_acc[(N1 * k + l) * NN + n] = acc;
-                        const Real cl = (Real)L.c[l];
-                        a0 += acc;
-                        a2 = fma(cl, acc, a2);
-                        a3 = fma(fma(ck, ck, cl * cl), acc, a3);
+                        if constexpr (KS == 1) add_moments(L, k, l, acc, m0, m1, m2, m3);
                     }
-                }
-#pragma unroll
-                for (int i = 0; i < KS; ++i) {
-                    if (k0 + i >= N1) break;
-                    const int from = i * (32 / KS) + lane % (32 / KS);
-                    const Real b0 = KS == 1 ? a0 : __shfl_sync(FULL, a0, from);
-                    m0 += b0;
-                    m1 = fma(KS == 1 ? ck : (Real)L.c[k0 + i], b0, m1);
-                    m2 += KS == 1 ? a2 : __shfl_sync(FULL, a2, from);
-                    m3 += KS == 1 ? a3 : __shfl_sync(FULL, a3, from);
                 }
             }
             if constexpr (KS > 1) {
 #pragma unroll
                 for (int o = 32 / KS; o < 32; o <<= 1) offwin |= __shfl_xor_sync(FULL, offwin, o);
+                // the moments in the order of one lane (another order shifts the
+                // rounding of a uniform flow the same way at every node and
+                // step: twice the error in u_y far from a vortex)
+                __syncwarp();
+                if (work) {
+#pragma unroll
+                    for (int q = 0; q < N1 * N1; ++q)
+                        add_moments(L, q / N1, q % N1, s_acc[q * NN + n], m0, m1, m2, m3);
+                }
+                __syncwarp();
             }
             // populations whose stencil leaves the staged window, from
             // global memory (outside the sweep, so the sweep keeps its
@@ -703,11 +708,7 @@ k_step_staged(StagedArgs<typename Tr::Real> A) {
                 const Real acc = staged_fallback<Tr, N1>(A, G, base, X, Y, k, l, pg.ux, pg.uy, pg.st);
                 if (part == 0) ++fallbacks;
                 s_acc[q * NN + n] = acc;
-                const Real ck = (Real)L.c[k], cl = (Real)L.c[l];
-                m0 += acc;
-                m1 = fma(ck, acc, m1);
-                m2 = fma(cl, acc, m2);
-                m3 = fma(fma(ck, ck, cl * cl), acc, m3);
+                add_moments(L, k, l, acc, m0, m1, m2, m3);
             }
             if (work) done = Tr::update(A.P, pg, m0, m1, m2, m3);
         }
